@@ -197,6 +197,10 @@ cudaError_t product_tc_jobs(const TcJobDesc* jobs, int njobs, void* dev_table, b
                             u32* err, int timeout_ms, cudaStream_t st, int* launches, int tile_n = 256,
                             bool diag_only = false);
 bool product_tc_supported(int device);
+// Clock ticks of timeout_ms at the current device's maximum clock: the bound of
+// the tensor-core kernels' waits.  The clock is asked of the driver once per
+// device: the query takes 0.36 ms, longer than many of the kernels it bounds.
+long long wait_budget(int timeout_ms);
 
 // ---- query.cu (serving) ---------------------------------------------------------
 // A resident reference index: the reference as one batch over [lo, lo+width)

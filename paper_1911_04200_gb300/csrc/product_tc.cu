@@ -41,6 +41,7 @@
 // budget, plus a CTA-wide abort flag); on time-out the CTA raises the error
 // word, waits (bounded) for its issued MMAs, frees its TMEM and leaves.
 #include <algorithm>
+#include <atomic>
 #include <vector>
 #include "common.cuh"
 #include "product_tc_sched.cuh"
@@ -517,15 +518,6 @@ k_prod_tc(const TcJobs P, u32* err, long long budget)
     }
 }
 
-long long wait_budget(int timeout_ms)
-{
-    int clk_khz = 0;
-    int clk_dev = 0;
-    cudaGetDevice(&clk_dev);
-    cudaDeviceGetAttribute(&clk_khz, cudaDevAttrClockRate, clk_dev);
-    return (long long)(clk_khz > 0 ? clk_khz : 2000000) * 1000LL * (long long)timeout_ms / 1000LL;
-}
-
 template <typename CT, int TN, bool DG = false, int SB = kStageBits>
 cudaError_t launch(const TcJobs& P, int sms, u32* err, int timeout_ms, cudaStream_t st)
 {
@@ -585,8 +577,21 @@ cudaError_t product_tc_jobs(const TcJobDesc* jobs, int njobs, void* dev_table, b
     return cudaSuccess;
 }
 
-namespace {
-}  // namespace
+long long wait_budget(int timeout_ms)
+{
+    static std::atomic<int> khz_by_dev[kMaxDevices];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    int khz = dev < kMaxDevices ? khz_by_dev[dev].load(std::memory_order_relaxed) : 0;
+    if (khz == 0) {
+        if (cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev) != cudaSuccess || khz <= 0) {
+            cudaGetLastError();
+            khz = 2000000;
+        }
+        if (dev < kMaxDevices) khz_by_dev[dev].store(khz, std::memory_order_relaxed);
+    }
+    return (long long)khz * (long long)timeout_ms;
+}
 
 bool product_tc_supported(int device)
 {

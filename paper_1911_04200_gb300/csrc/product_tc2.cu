@@ -813,11 +813,8 @@ cudaError_t run(ProductArgs& a, const CUtensorMap& map, cudaStream_t st)
         if (dev < kMaxDevices) resident_by_dev[dev].store(nc, std::memory_order_relaxed);
     }
     const u64 clusters = std::min<u64>((u64)std::min(resident, a.sms / 2), total);
-    int clk_khz = 0;
-    cudaDeviceGetAttribute(&clk_khz, cudaDevAttrClockRate, dev);
-    long long budget = (long long)(clk_khz > 0 ? clk_khz : 2000000) * 1000LL * (long long)a.timeout_ms / 1000LL;
     k_prod_tc2<CT, TMA><<<(unsigned)(2 * clusters), kThreads, kSmemBytes, st>>>(map, a.X, a.stride, a.n, a.W, tiles, L,
-                                                                          (CT*)a.C, a.ldc, a.err, budget);
+                                                                          (CT*)a.C, a.ldc, a.err, wait_budget(a.timeout_ms));
     a.launches += 1;
     return cudaGetLastError();
 }
