@@ -65,40 +65,36 @@ cudaError_t launch_feed_piece(const u64* hv, u64* dv, const u64* off, u64 n, con
 // ---- windows.cu ------------------------------------------------------------
 // Windowed ingest of the block-sparse path: the batch [lo, lo + nwin 2^wl)
 // of a plan over n samples in tile order (tiles of 128) is cut into nwin
-// windows of 2^wl rows, and the windows into G ranges of wpc (the last one
-// possibly shorter); both passes run one CTA per (range, tile).
-// A range holds at most kWinRangeWords words (of 64 rows) per class: pass 2
-// keeps two classes' words of a range in shared memory.
-constexpr u64 kMaxWinPerRange = 16;
-constexpr u64 kWinRangeWords = 4096;
+// windows of 2^wl rows.  Pass 1 runs one CTA per (group of gw windows, tile),
+// pass 2 one per (range of wpc windows, tile); the last group or range may be
+// shorter.  A group is whole ranges.
+constexpr u64 kMaxWinPerRange = 2;
 struct WinGeom {
     u64 n, T, lo;
-    u64 nwin, wpc, G;
-    u64 nw;     // words per class bitmap: nwin 2^wl / 64
-    int wl;     // log2 of the rows of a window, 12..16
-    // per tile, the order its samples are handed to warps (tile-local
-    // positions, largest sample first: entry 128t + j of the plan's order)
-    const u32* lpt;
+    u64 nwin, wpc, G;   // windows; windows per range; ranges
+    u64 gw, NG;         // windows per group; groups
+    u64 nw;             // words per class bitmap: nwin 2^wl / 64
+    int wl, wpc_log;    // log2 of the rows of a window, 12..16, and of wpc
 };
+// The windows, ranges and groups of the batch [lo, lo + width) (width a
+// multiple of 2^wl).
+WinGeom win_geom(u64 n, u64 T, u64 lo, u64 width, int wl, bool twice);
 // Pass 1: B (B2 with the two-or-more filter; T x nw words, tile-major) = the
 // tiles' filter bitmaps, cls ((T + 1) x nw, class-major) = the class
 // bitmaps, pre (likewise) = every class word's rank within its window (the
 // class's rows of the window below the word), cnt ((T + 1) x nwin) = every
-// window's rows per class, agg
-// ((T + 1) x G) = every range's rows per class rounded up to 64, curs
-// ((G + 1) x n) = every sample's position at each range start and at the
-// batch end; plan.totals[kPlanRowsTotal] += the rows of all classes (zeroed
-// by the plan).
-size_t win_tiles_smem(const WinGeom& g, bool twice);
-cudaError_t launch_win_classes(const u64* ids, Plan plan, const WinGeom& g, bool twice, u64* B, u64* B2, u64* cls,
-                               unsigned short* pre, u32* cnt, u64* agg, u64* curs, cudaStream_t st);
+// window's rows per class, agg ((T + 1) x G) = every range's rows per class
+// rounded up to 64, gcurs ((NG + 1) x n) = every sample's position at each
+// group start and at the batch end, curs ((G + 1) x n) = at each range start;
+// plan.totals[kPlanRowsTotal] += the rows of all classes (zeroed by the plan).
+cudaError_t launch_win_classes(const u64* ids, u64 N, Plan plan, const WinGeom& g, bool twice, u64* B, u64* B2, u64* cls,
+                               unsigned short* pre, u32* cnt, u64* agg, u64* gcurs, u64* curs, cudaStream_t st);
 // Pass 2: with boff the exclusive prefix of agg (class c's range r at
 // boff[c G + r] - boff[c G]), every word of the batch's class-0 part of XM
 // (words [kbase[0], kbase[0] + W_0) of rows 0..n-1; null: no class-0 rows)
 // and of tile t's part of XS (words [kbase[1 + t], ...) of rows 128t..) is
 // stored once, with plain stores.
-size_t win_pack_smem(const WinGeom& g);
-cudaError_t launch_win_pack(const u64* ids, const WinGeom& g, const u64* cls, const unsigned short* pre,
+cudaError_t launch_win_pack(const u64* ids, u64 N, const WinGeom& g, const u64* cls, const unsigned short* pre,
                             const u32* cnt, const u64* boff, const u64* curs, const u64* kbase, u64* XM, u64 stride_m,
                             u64* XS, u64 stride_s, cudaStream_t st);
 

@@ -228,7 +228,7 @@ u64 sparse_batch_rows(const jsim_ctx* ctx, u64 n, u64 span, bool windowed = fals
         if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) { cudaGetLastError(); return kMinClassRows; }
         auto slots_bytes = [&](u64 m) {
             const u64 nwin = m >> kWinLog;
-            return 2 * (m / 8 * (T * f2 + T + 1) + m / 64 * 2 * (T + 1) + (nwin + 1) * n * 8 + (T + 1) * nwin * 12);
+            return 2 * (m / 8 * (T * f2 + T + 1) + m / 64 * 2 * (T + 1) + (nwin / 2 + nwin / 4 + 2) * n * 8 + (T + 1) * nwin * 12);
         };
         while (mt > kMinClassRows && (slots_bytes(mt) > total_b / 16 || slots_bytes(mt) > free_b / 4)) mt >>= 1;
         return mt;
@@ -274,19 +274,6 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
     const u64 mt = feed ? feed->mt : sparse_batch_rows(ctx, n, span, windowed);
     if (!mt) return JSIM_ERR_UNSUPPORTED;
     ctx->stats.batch_rows = mt;
-    auto geom = [&](u64 lo, u64 width) {
-        WinGeom g{};
-        g.n = n;
-        g.T = T;
-        g.lo = lo;
-        g.wl = wl;
-        g.nwin = width >> wl;
-        g.nw = width / 64;
-        g.wpc = std::min<u64>(std::max<u64>(g.nwin, 1), std::min<u64>(kMaxWinPerRange, kWinRangeWords >> (wl - 6)));
-        g.G = (g.nwin + g.wpc - 1) / g.wpc;
-        return g;
-    };
-
     // search bounds of a batch at lo: with a feed, the slices of lo's piece
     const u64* pb = st.d_off;
     const u64* pe = nullptr;
@@ -304,7 +291,7 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
     // kSketchPerSample per sample ----
     std::vector<u32> order(n), pos(n);
     for (u64 i = 0; i < n; ++i) order[i] = (u32)i;
-    DevBuf d_pos, d_order, d_tile, d_cls_of, d_rowk, d_lpt, jobtab, Wc, kbase;
+    DevBuf d_pos, d_order, d_tile, d_cls_of, d_rowk, jobtab, Wc, kbase;
     const u64 nw_max = mt / 64;
     const u64 nb_max = (T + 1) * nw_max / kScanBlockWords;
     // Two slots of batch structures: the next batch is classified while this
@@ -314,7 +301,7 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
     // bases from [128 + 64 s, +2(T + 1)).  Windowed: bsum holds the ranges'
     // rows per class, cnt the windows', curs the window-start cursors.
     struct Slot {
-        DevBuf B, B2, cls, dir, bsum, boff, Rd, plan_buf, cnt, curs, pre;
+        DevBuf B, B2, cls, dir, bsum, boff, Rd, plan_buf, cnt, curs, gcurs, pre;
         Plan plan{};
         WinGeom g{};
         cudaEvent_t done = nullptr;    // totals on the host
@@ -337,7 +324,9 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
             ALLOC(x.pre, (T + 1) * nw_max * sizeof(unsigned short));
             ALLOC(x.bsum, (T + 1) * ranges_max * sizeof(u64));
             ALLOC(x.boff, ((T + 1) * ranges_max + 1) * sizeof(u64));
-            ALLOC(x.curs, (nwin_max + 1) * n * sizeof(u64));
+            const WinGeom wg = win_geom(n, T, 0, mt, wl, twice);
+            ALLOC(x.curs, (wg.G + 1) * n * sizeof(u64));
+            ALLOC(x.gcurs, (wg.NG + 1) * n * sizeof(u64));
         } else {
             ALLOC(x.B, T * nw_max * sizeof(u64));
             if (twice) ALLOC(x.B2, T * nw_max * sizeof(u64));
@@ -391,7 +380,6 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
     ALLOC(d_pos, n * sizeof(u32));
     ALLOC(d_order, n * sizeof(u32));
     ALLOC(d_rowk, n * sizeof(u32));
-    ALLOC(d_lpt, n * sizeof(u32));
     ALLOC(d_tile, n * sizeof(u32));
     ALLOC(d_cls_of, n * sizeof(u32));
     ALLOC(jobtab, kMaxTiles * sizeof(TcJobDesc));
@@ -405,18 +393,17 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
         const u64 hi = lo + width;  // 0 on wrap-around: unbounded
         u64* hs = ctx->h_scalars + 64 + 32 * si;
         if (windowed) {
-            x.g = geom(lo, width);
-            x.g.lpt = d_lpt.as<u32>();
+            x.g = win_geom(n, T, lo, width, wl, twice);
             if (x.g.nwin > nwin_max || x.g.G > ranges_max || x.g.nwin * (1ull << wl) != width)
                 return JSIM_ERR_UNSUPPORTED;  // the slot's buffers are sized for nwin_max windows
             if (x.pack_pending) CK(cudaStreamWaitEvent(ccs, x.packed, 0));
             {
                 StageTimer t(ctx, &ctx->stats.ms_filter, ccs);
                 CK(launch_plan(pb, st.d_ids, n, lo, hi, false, x.plan, ccs, d_order.as<u32>(), pe));
-                CK(launch_win_classes(st.d_ids, x.plan, x.g, twice, x.B.as<u64>(), twice ? x.B2.as<u64>() : nullptr,
+                CK(launch_win_classes(st.d_ids, st.N, x.plan, x.g, twice, x.B.as<u64>(), twice ? x.B2.as<u64>() : nullptr,
                                       x.cls.as<u64>(), x.pre.as<unsigned short>(), x.cnt.as<u32>(),
-                                      x.bsum.as<u64>(), x.curs.as<u64>(), ccs));
-                ctx->stats.launches += 4;
+                                      x.bsum.as<u64>(), x.gcurs.as<u64>(), x.curs.as<u64>(), ccs));
+                ctx->stats.launches += 5;
                 ctx->stats.windows += x.g.nwin;
             }
             {
@@ -484,7 +471,6 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
         return JSIM_OK;
     };
 
-    std::vector<u64> ssz(n, 0);  // the samples' sketch sizes (by sample)
     if (st.N) {
         u64 ws = 1ull << 16;
         const double want = (double)kSketchPerSample * (double)n;
@@ -534,26 +520,15 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
             CK(cudaStreamSynchronize(cs));
             const u64* h_sz = (const u64*)ctx->h_sketch;
             order = sample_order((const float*)(h_sz + n), h_sz, n);
-            ssz.assign(h_sz, h_sz + n);
         }
         for (u64 k = 0; k < n; ++k) pos[order[k]] = (u32)k;
-        // per plan entry k (the sample at position k): its tile, class and
-        // row; and per tile the order its samples go to the windowed kernels'
-        // warps: largest sketch first (sizes vary by two decades, and a large
-        // sample taken last would hold its CTA up)
-        std::vector<u32> tile(n), cls_of(n), rowk(n), lpt(n);
+        // per plan entry k (the sample at position k): its tile, class and row
+        std::vector<u32> tile(n), cls_of(n), rowk(n);
         for (u64 k = 0; k < n; ++k) {
             tile[k] = (u32)(k / kTile);
             cls_of[k] = 1 + tile[k];
             rowk[k] = (u32)k;
-            lpt[k] = (u32)(k % kTile);
         }
-        for (u64 k0 = 0; k0 < n; k0 += kTile) {
-            u32* l = lpt.data() + k0;
-            const u64 m = std::min<u64>(kTile, n - k0);
-            std::stable_sort(l, l + m, [&](u32 a, u32 b) { return ssz[order[k0 + a]] > ssz[order[k0 + b]]; });
-        }
-        CK(cudaMemcpyAsync(d_lpt.p, lpt.data(), n * sizeof(u32), cudaMemcpyHostToDevice, cs));
         CK(cudaMemcpyAsync(d_pos.p, pos.data(), n * sizeof(u32), cudaMemcpyHostToDevice, cs));
         CK(cudaMemcpyAsync(d_order.p, order.data(), n * sizeof(u32), cudaMemcpyHostToDevice, cs));
         CK(cudaMemcpyAsync(d_tile.p, tile.data(), n * sizeof(u32), cudaMemcpyHostToDevice, cs));
@@ -729,7 +704,7 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
                 if (windowed) {
                     StageTimer t(ctx, &ctx->stats.ms_pack);
                     CK(cudaStreamWaitEvent(cs, x.done, 0));
-                    CK(launch_win_pack(st.d_ids, x.g, x.cls.as<u64>(), x.pre.as<unsigned short>(), x.cnt.as<u32>(),
+                    CK(launch_win_pack(st.d_ids, st.N, x.g, x.cls.as<u64>(), x.pre.as<unsigned short>(), x.cnt.as<u32>(),
                                        x.boff.as<u64>(), x.curs.as<u64>(), kbase.as<u64>(),
                                        W[0] ? XM.as<u64>() : nullptr, stride_m, Wmax_s ? XS.as<u64>() : nullptr,
                                        stride_s, cs));

@@ -3,13 +3,28 @@
 // ranks (Eq. 6) and the bitmask compression (Sec. III-B), built range by
 // range in shared memory.
 //
-// A row batch [lo, lo + m) is cut into windows of 2^wl rows and the windows
-// into ranges of up to wpc consecutive windows.  A sample's values are
-// sorted, so a sample's values in a range are one segment, walked by one
-// warp; its start is found by binary search once per group of ranges.
+// A row batch [lo, lo + m) is cut into windows of 2^wl rows.  A sample's
+// values are sorted, so its values in a run of rows are one segment.  Set
+// sizes vary by two decades, so both passes treat the segments of a tile's
+// samples in their run of rows as one flat list of aligned 32-byte pieces of
+// four values, split evenly over the warps, one piece a lane and step: a
+// lane's position tells its sample (the segments' running starts lie in
+// shared memory), no lane idles on a short segment, every load is one full
+// sector, and nothing is paid per sample but its two cursors.  What bounds
+// them (1024 clade samples, 1.3e9 values, 20 values a sample and window of
+// 2^16 rows): pass 1 instruction issue (62 % of slots) at 4.0 TB/s; pass 2
+// the shared-memory pipe (57 %) and the barriers between its phases, at 2.7
+// TB/s.  Measured on the whole call, ms: a warp per sample and range 5.9 +
+// 13.0 (passes 1 and 2); a flat list of single values 6.5 + 11.8; runs of
+// four values a lane, loaded word by word 5.0 + 12.2; aligned pieces in one
+// 32-byte load 3.9 + 9.9, with 1.4 for the cursors.  Ranges of 1, 2 and 4
+// windows in pass 2 take 10.6, 9.9 and 10.4; three CTAs an SM of pass 1 cost
+// more in registers than they hide (4.9).
 //
-// Pass 1 (k_win_tiles, one CTA per group of kTileRanges ranges and tile):
-// the tile's filter bitmap of each range is set in shared memory and stored.
+// k_win_cursors: every sample's position at each group of windows.  Pass 1
+// (k_win_tiles, one CTA per group and tile): the tile's filter bitmap of the
+// group is set in shared memory and stored, and every sample's position at
+// each range of pass 2 noted where its values cross into the range.
 // k_win_classify (one CTA per window) classifies the rows - class 0: held by
 // two or more tiles; class 1 + t: by tile t alone (with the two-or-more
 // filter, by two or more of its samples) - and writes every class word's
@@ -23,10 +38,10 @@
 //
 // Pass 2 (k_win_pack, one CTA per range and tile): the tile's samples are
 // packed into the class-0 matrix XM and the tile's matrix XS.  A value's
-// class and rank come from the range's class words and their window ranks
-// in shared memory; a sample's bits are gathered in shared memory, kStage
-// words at a time, and stored as whole words with plain stores.  Every word
-// of the batch's part of XM and XS is written exactly once, zero words
+// class and rank come from the range's class words and ranks in shared
+// memory; the words of a group of samples (as many as fit, usually the whole
+// tile) are gathered there too and stored whole with plain stores.  Every
+// word of the batch's part of XM and XS is written exactly once, zero words
 // included, so nothing is zeroed beforehand and no global atomics are
 // needed.
 #include "ingest_dev.cuh"
@@ -35,152 +50,294 @@ namespace jsim {
 
 namespace {
 
-constexpr int kWin1Threads = 256;
-constexpr int kSlots1 = 4;        // samples a warp walks at once in pass 1
-constexpr int kClassThreads = 256;
-constexpr int kClassWords = 4;    // words of a window per classify thread (2^16 rows = 256 x 4 words)
-constexpr u64 kTileRanges = 4;    // consecutive ranges a pass-1 CTA walks
-constexpr int kWin2Threads = 512;
-constexpr int kWin2Warps = kWin2Threads / 32;
-constexpr int kDepth2 = 4;        // 32-value chunks of a sample a warp loads at once in pass 2
-constexpr int kStage = 64;        // words gathered at a time per sample and class
+constexpr int kWinThreads = 512;
+constexpr u32 kRun = 4;           // values a lane takes at a time: 32 aligned bytes
+constexpr int kClassThreads = 512;
+constexpr int kCursChunk = 8;     // consecutive cursors a thread of k_win_cursors finds
 constexpr u64 kWinTile = 128;     // samples per tile
+constexpr u32 kRoundLen = 1u << 24;     // values of a segment listed at a time (128 of them fit 32-bit positions)
+constexpr u32 kStageWords = 5120;       // words gathered at a time in pass 2 (40 KiB)
 
-// Bring the 32 values from p on (up to e) toward L2 ahead of their loads.
-__device__ __forceinline__ void prefetch_values(const u64* ids, u64 p, u64 e)
+// The values as 32-byte pieces: piece p is ids[4 p - ph .. 4 p - ph + 3], ph
+// the values that ids lies past a 32-byte boundary.
+struct Values {
+    const u64* ids;
+    u64 n;
+    u32 ph;
+};
+
+// The flat list of up to 128 segments [a, b) of ids, in pieces (a segment's
+// first and last piece may hold other values too): segment k's pieces are
+// list entries [start[k], start[k + 1]).
+struct PieceList {
+    u64 a[kWinTile], b[kWinTile];
+    u32 start[kWinTile + 1];
+    u32 scan[kWinTile / 32];
+};
+
+// Lists values [r kRoundLen, (r + 1) kRoundLen) of every segment whose thread
+// (0 .. 127) has a < b; returns the list's length.  All threads call; the
+// list may be read after it, and rebuilt after a barrier.
+__device__ __forceinline__ u32 list_build(PieceList& L, const Values& v, u64 a, u64 b, u32 r)
 {
-    if (p < e) asm volatile("prefetch.global.L2 [%0];" ::"l"(ids + p));
-    if (p + 16 < e) asm volatile("prefetch.global.L2 [%0];" ::"l"(ids + p + 16));
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    u32 runs = 0, inc = 0;
+    if (tid < (int)kWinTile) {
+        a = min(b, a + (u64)r * kRoundLen);
+        b = min(b, a + kRoundLen);
+        runs = a < b ? (u32)(((b - 1 + v.ph) >> 2) - ((a + v.ph) >> 2)) + 1 : 0;
+        inc = runs;
+        #pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const u32 y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane == 31) L.scan[warp] = inc;
+        L.a[tid] = a;
+        L.b[tid] = b;
+    }
+    __syncthreads();
+    u32 total = 0, before = 0;
+    #pragma unroll
+    for (int w = 0; w < (int)kWinTile / 32; ++w) {
+        if (w < warp) before += L.scan[w];
+        total += L.scan[w];
+    }
+    if (tid < (int)kWinTile) L.start[tid] = before + inc - runs;
+    if (tid == 0) L.start[kWinTile] = total;
+    __syncthreads();
+    return total;
 }
 
-// Pass 1: CTA (range group rq, tile t) = blockIdx.x (rq * T + t) walks
-// tile t's samples through ranges kTileRanges rq .. kTileRanges rq +
-// kTileRanges - 1 in turn: per range it sets the rows that the tile's
-// samples hold (Eq. 5 over the tile; TWICE: also the rows two or more of
-// them hold) in shared memory and stores the bitmaps to B (and B2),
-// tile-major.  Only the group's first range needs its cursors found by
-// search; the next range starts where the walk stopped.  Shared memory: the
-// bitmaps, then the tile's cursors and ends.  A warp walks kSlots1 samples
-// at once, 32 consecutive values of each per step, and takes the next
-// sample when one leaves the range.  Five CTAs an SM with one filter bitmap
-// (47 registers, no spills); the two-or-more filter keeps four.
+// A lane's walk through a list, forward: its piece's segment k, the value
+// index of its first word (negative for a piece that begins before ids) and
+// the words [lo, hi) of it that belong to the segment.
+struct Walk {
+    u32 k, beg, end, b, skip;  // segment; its list positions; low word of its end; words before it in its first piece
+    long long off;             // the segment's piece at list position f is off + f
+    long long base;
+    u32 lo, hi;
+    __device__ __forceinline__ void load(const PieceList& L, const Values& v)
+    {
+        beg = L.start[k];
+        end = L.start[k + 1];
+        const u64 sa = L.a[k] + v.ph;
+        skip = (u32)sa & 3u;
+        off = (long long)(sa >> 2) - (long long)beg;
+        b = (u32)L.b[k];
+    }
+    // at list position f (below the list's length)
+    __device__ __forceinline__ void init(const PieceList& L, const Values& v, u32 f)
+    {
+        u32 l = 0, h = kWinTile - 1;
+        while (l < h) {
+            const u32 mid = (l + h + 1) >> 1;
+            if (L.start[mid] <= f) l = mid; else h = mid - 1;
+        }
+        k = l;
+        load(L, v);
+    }
+    __device__ __forceinline__ void to(const PieceList& L, const Values& v, u32 f)
+    {
+        if (f >= end) {
+            do ++k; while (f >= L.start[k + 1]);
+            load(L, v);
+        }
+        base = 4 * (off + f) - (long long)v.ph;
+        lo = f == beg ? skip : 0;
+        hi = min(kRun, b - (u32)base);
+    }
+};
+
+// The low words of a piece's four values (a piece at either end of ids is
+// read value by value).
+__device__ __forceinline__ void load_piece(const Values& v, const Walk& w, u32 (&x)[kRun])
+{
+    if (w.base >= 0 && w.base + (long long)kRun <= (long long)v.n) {
+        u64 y[kRun];
+        asm volatile("ld.global.nc.v4.u64 {%0,%1,%2,%3}, [%4];\n"
+                     : "=l"(y[0]), "=l"(y[1]), "=l"(y[2]), "=l"(y[3]) : "l"(v.ids + w.base));
+        #pragma unroll
+        for (u32 i = 0; i < kRun; ++i) x[i] = (u32)y[i];
+    } else {
+        #pragma unroll
+        for (u32 i = 0; i < kRun; ++i) x[i] = i >= w.lo && i < w.hi ? (u32)v.ids[w.base + i] : 0u;
+    }
+}
+
+// Rows of a piece's values: those outside [lo, hi) take the nearest one
+// inside (a bit set twice is set once).
+__device__ __forceinline__ void rows_of(u32 (&x)[kRun], u32 lo, u32 hi, u32 origin, u32 mask)
+{
+    #pragma unroll
+    for (u32 i = 0; i < kRun; ++i) x[i] = (x[i] - origin) & mask;
+    #pragma unroll
+    for (int i = (int)kRun - 2; i >= 0; --i) x[i] = (u32)i < lo ? x[i + 1] : x[i];
+    #pragma unroll
+    for (u32 i = 1; i < kRun; ++i) x[i] = i >= hi ? x[i - 1] : x[i];
+}
+
+// Every sample's position at the start of each group of g.gw windows (and at
+// the batch end): gcurs[g n + k] for entry k of the plan.  A thread bisects
+// for its first group and gallops on from there, by the sample's mean
+// distance.
+__global__ void k_win_cursors(const u64* __restrict__ ids, Plan plan, WinGeom g, u64* __restrict__ gcurs)
+{
+    const u32 i = blockIdx.x * blockDim.x + threadIdx.x, c = i / (u32)g.n, k = i - c * (u32)g.n;
+    const u64 g0 = (u64)c * kCursChunk, g1 = min(g0 + kCursChunk, g.NG);
+    if (g0 >= g.NG) return;
+    const u64 b = plan.beg[k], e = b + plan.len[k];
+    const u64 mean = (e - b) / g.NG + 1;
+    u64 pos = b;
+    for (u64 gi = g0; gi < g1; ++gi) {
+        const u64 bound = g.lo + ((gi * g.gw) << g.wl);
+        if (gi == g0) {
+            pos = gi ? lower_bound_u64(ids, b, e, bound) : b;
+        } else {
+            // from the expected place outward in steps of a sector, then 2, 4 .. of them
+            u64 lo = pos, hi = min(e, pos + mean), step = 4;
+            if (hi < e && ids[hi] < bound) {
+                do {
+                    lo = hi + 1;
+                    hi = min(e, lo + step);
+                    step *= 2;
+                } while (hi < e && ids[hi] < bound);
+            } else {
+                while (hi > lo + step && ids[hi - step] >= bound) {
+                    hi -= step;
+                    step *= 2;
+                }
+                if (hi > lo + step) lo = hi - step;
+            }
+            pos = lower_bound_u64(ids, lo, hi, bound);
+        }
+        gcurs[gi * g.n + k] = pos;
+    }
+    if (g1 == g.NG) gcurs[g.NG * g.n + k] = e;
+}
+
+// Pass 1: CTA (group gi, tile t) = blockIdx.x (gi * T + t) sets the rows that
+// tile t's samples hold in the group's windows (Eq. 5 over the tile; TWICE:
+// also the rows two or more of them hold) in shared memory and stores the
+// bitmaps to B (and B2), tile-major.  curs gets every sample's position at
+// the start of each pass-2 range.  Shared memory: the bitmaps (64 KiB: groups
+// of 8 windows, 4 with TWICE), then the list.
 template <bool TWICE>
-__global__ void __launch_bounds__(kWin1Threads, TWICE ? 4 : 5)
-k_win_tiles(const u64* __restrict__ ids, Plan plan, WinGeom g, u64* __restrict__ B, u64* __restrict__ B2,
-            u64* __restrict__ curs)
+__global__ void __launch_bounds__(kWinThreads, 2)
+k_win_tiles(Values v, WinGeom g, const u64* __restrict__ gcurs, u64* __restrict__ B,
+            u64* __restrict__ B2, u64* __restrict__ curs)
 {
     extern __shared__ __align__(16) unsigned char win_smem[];
-    const u64 rq = blockIdx.x / g.T, t = blockIdx.x % g.T;
+    const u32 gi = blockIdx.x / (u32)g.T, t = blockIdx.x - gi * (u32)g.T;
+    const u64 w0 = gi * g.gw, w1 = min(w0 + g.gw, g.nwin);
+    const u64 rows = (w1 - w0) << g.wl;
+    const u32 glo32 = (u32)(g.lo + (w0 << g.wl));
     u32* bm = reinterpret_cast<u32*>(win_smem);
-    u32* bm2 = bm + (g.wpc << (g.wl - 5));
-    u64* cur = reinterpret_cast<u64*>(bm + (TWICE ? 2 : 1) * (g.wpc << (g.wl - 5)));
-    u64* cend = cur + kWinTile;
-    __shared__ u32 s_next;
-    const int tid = threadIdx.x, lane = tid & 31;
+    u32* bm2 = bm + (g.gw << (g.wl - 5));
+    PieceList& L = *reinterpret_cast<PieceList*>(bm + (TWICE ? 2 : 1) * (g.gw << (g.wl - 5)));
+    __shared__ u32 s_rounds;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const u64 k0 = t * kWinTile, m = min(kWinTile, g.n - k0);
-    const u64 r_end = min(rq * kTileRanges + kTileRanges, g.G);
+    // pass-2 ranges of the group: r0 on; a row of the group >> rsh is its range
+    const u64 r0 = w0 >> g.wpc_log;
+    const u32 nr = (u32)((w1 - w0 + g.wpc - 1) >> g.wpc_log);
+    const int rsh = g.wl + g.wpc_log;
 
-    for (u64 r = rq * kTileRanges; r < r_end; ++r) {
-        const u64 w0 = r * g.wpc, w1 = min(w0 + g.wpc, g.nwin);
-        const u64 rows_r = (w1 - w0) << g.wl, RW64 = rows_r >> 6;
-        const u64 rlo = g.lo + (w0 << g.wl);
-        {
-            uint4* z = reinterpret_cast<uint4*>(bm);
-            const u64 nz = (TWICE ? 2 : 1) * (g.wpc << (g.wl - 5)) / 4;
-            for (u64 i = tid; i < nz; i += kWin1Threads) z[i] = make_uint4(0u, 0u, 0u, 0u);
-        }
-        if (tid == 0) s_next = 0;
-        for (u64 kk = tid; kk < m; kk += kWin1Threads) {
-            u64 c;
-            if (r == rq * kTileRanges) {
-                const u64 b = plan.beg[k0 + kk], e = b + plan.len[k0 + kk];
-                c = w0 == 0 ? b : lower_bound_u64(ids, b, e, rlo);
-                cur[kk] = c;
-                cend[kk] = e;
-            } else {
-                c = cur[kk];
-            }
-            curs[r * g.n + k0 + kk] = c;
-        }
-        __syncthreads();
-        for (u64 kk = tid; kk < m; kk += kWin1Threads) prefetch_values(ids, cur[kk], cend[kk]);
-
-        // samples go to warps as they free a slot (sizes vary by two decades)
-        u64 ks[kSlots1], ps[kSlots1], es[kSlots1], prev[kSlots1];
-        bool act[kSlots1], hp[kSlots1];
-        auto take = [&](int s) {
-            u32 e = 0;
-            if (lane == 0) {
-                e = atomicAdd(&s_next, 1u);
-                if (e < m) e = g.lpt[k0 + e];  // largest samples first
-            }
-            e = __shfl_sync(0xffffffffu, e, 0);
-            act[s] = e < m;
-            ks[s] = e;
-            ps[s] = act[s] ? cur[e] : 0;
-            es[s] = act[s] ? cend[e] : 0;
-            hp[s] = false;  // the value before a range's first one is below it (sorted input)
-            prev[s] = 0;
-        };
-        #pragma unroll
-        for (int s = 0; s < kSlots1; ++s) take(s);
-        for (;;) {
-            bool any = false;
-            #pragma unroll
-            for (int s = 0; s < kSlots1; ++s) any = any || act[s];
-            if (!any) break;
-            u64 x[kSlots1];
-            #pragma unroll
-            for (int s = 0; s < kSlots1; ++s) {
-                const u64 pos = ps[s] + (u64)lane;
-                x[s] = (act[s] && pos < es[s]) ? ids[pos] : 0ull;
-            }
-            #pragma unroll
-            for (int s = 0; s < kSlots1; ++s) {
-                if (!act[s]) continue;
-                const u64 pos = ps[s] + (u64)lane, v = x[s], d = v - rlo;
-                // the values from the first one at or past the range's end stay for
-                // the next range (a value below it only comes from unsorted input,
-                // and is passed over)
-                const bool stop = pos >= es[s] || (v >= rlo && d >= rows_r);
-                const unsigned bal = __ballot_sync(0xffffffffu, stop);
-                const int run = bal ? __ffs((int)bal) - 1 : 32;
-                if (TWICE) {
-                    const u64 pv = __shfl_up_sync(0xffffffffu, v, 1);
-                    const u64 lastv = __shfl_sync(0xffffffffu, v, 31);
-                    const bool dup = lane ? pv == v : (hp[s] && prev[s] == v);
-                    if (lane < run && v >= rlo && !dup) {
-                        const u32 bit = 1u << (d & 31);
-                        const u32 old = atomicOr(bm + (d >> 5), bit);
-                        if (old & bit) atomicOr(bm2 + (d >> 5), bit);
+    {
+        uint4* z = reinterpret_cast<uint4*>(bm);
+        const u32 nz = (u32)((TWICE ? 2 : 1) * (g.gw << (g.wl - 5)) / 4);
+        for (u32 i = tid; i < nz; i += kWinThreads) z[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    if (tid == 0) s_rounds = 0;
+    __syncthreads();
+    u64 a = 0, b = 0;
+    if (tid < m) {
+        a = gcurs[gi * g.n + k0 + tid];
+        b = max(a, gcurs[(gi + 1) * g.n + k0 + tid]);
+        // the ranges no value crosses into start at the segment's end
+        curs[r0 * g.n + k0 + tid] = a;
+        for (u32 r = 1; r < nr; ++r) curs[(r0 + r) * g.n + k0 + tid] = b;
+        if (w1 == g.nwin) curs[g.G * g.n + k0 + tid] = b;
+        if (b > a) atomicMax(&s_rounds, (u32)((b - a + kRoundLen - 1) / kRoundLen));
+    }
+    __syncthreads();
+    const u32 rounds = s_rounds;
+    // Rows are taken modulo the bitmap: a row outside the group only comes
+    // from unsorted input, whose results are dropped.
+    const u32 mask = (u32)(g.gw << g.wl) - 1;
+    for (u32 rd = 0; rd < rounds; ++rd) {
+        const u32 F = list_build(L, v, a, b, rd);
+        const u32 cw = (F + kWinThreads - 1) / kWinThreads * 32;  // a warp's share: whole steps of a piece a lane
+        const u32 f0 = warp * cw, f1 = min(F, f0 + cw);
+        if (f0 < f1) {
+            Walk wk;
+            wk.init(L, v, min(f0 + lane, f1 - 1));
+            u32 nx[kRun];  // the next piece's values, loaded ahead
+            wk.to(L, v, min(f0 + lane, f1 - 1));
+            load_piece(v, wk, nx);
+            u32 cd = 0;    // the row before the step's first piece
+            if (lane == 0 && (f0 != wk.beg || rd > 0)) cd = ((u32)v.ids[wk.base + wk.lo - 1] - glo32) & mask;
+            for (u32 f = f0 + lane; f - lane < f1; f += 32) {
+                u32 x[kRun];
+                #pragma unroll
+                for (u32 i = 0; i < kRun; ++i) x[i] = nx[i];
+                rows_of(x, wk.lo, wk.hi, glo32, mask);
+                const u32 k = wk.k;
+                const u64 s = (u64)wk.base;
+                const u32 lo = wk.lo;
+                const bool in = f < f1;
+                // the row before the piece, if it is of the sample's segment of the
+                // group (else 0: the first range's start)
+                const bool first = f == wk.beg;
+                u32 pd = __shfl_up_sync(0xffffffffu, x[kRun - 1], 1);
+                if (lane == 0) pd = cd;
+                cd = __shfl_sync(0xffffffffu, x[kRun - 1], 31);
+                bool prev = !first;
+                if (first) {
+                    pd = 0;
+                    if (rd > 0) {  // the list begins inside the segment
+                        pd = ((u32)v.ids[s + lo - 1] - glo32) & mask;
+                        prev = true;
                     }
-                    hp[s] = true;
-                    prev[s] = lastv;
-                } else if (lane < run && v >= rlo) {
-                    atomicOr(bm + (d >> 5), 1u << (d & 31));
                 }
-                ps[s] += (u64)run;
-                if (run < 32) {
-                    if (lane == 0) {
-                        cur[ks[s]] = ps[s];  // the next range of the group starts here
-                        // the last range's ends close pass 2's segments (every other
-                        // group's CTA finds its own first cursors)
-                        if (r + 1 == g.G) curs[(r + 1) * g.n + k0 + ks[s]] = ps[s];
+                if (f + 32 < f1) {
+                    wk.to(L, v, f + 32);
+                    load_piece(v, wk, nx);
+                }
+                if (!in) continue;
+                if ((x[kRun - 1] >> rsh) > (pd >> rsh)) {
+                    // the values cross into further ranges
+                    u32 pr = pd >> rsh;
+                    #pragma unroll
+                    for (u32 i = 0; i < kRun; ++i) {
+                        const u32 rg = min(x[i] >> rsh, nr - 1);
+                        for (; pr < rg; ++pr) curs[(r0 + pr + 1) * g.n + k0 + k] = s + max(i, lo);
                     }
-                    take(s);
+                }
+                #pragma unroll
+                for (u32 i = 0; i < kRun; ++i) {
+                    const u32 bit = 1u << (x[i] & 31);
+                    if (TWICE) {
+                        if (i ? x[i] != x[i - 1] : !prev || x[0] != pd) {
+                            const u32 old = atomicOr(bm + (x[i] >> 5), bit);
+                            if (old & bit) atomicOr(bm2 + (x[i] >> 5), bit);
+                        }
+                    } else {
+                        atomicOr(bm + (x[i] >> 5), bit);
+                    }
                 }
             }
         }
-        __syncthreads();
-        const u64* b64 = reinterpret_cast<const u64*>(bm);
-        u64* out = B + t * g.nw + (w0 << (g.wl - 6));
-        for (u64 j = tid; j < RW64; j += kWin1Threads) out[j] = b64[j];
-        if (TWICE) {
-            const u64* c64 = reinterpret_cast<const u64*>(bm2);
-            u64* out2 = B2 + t * g.nw + (w0 << (g.wl - 6));
-            for (u64 j = tid; j < RW64; j += kWin1Threads) out2[j] = c64[j];
-        }
-        __syncthreads();  // the bitmaps are cleared and the cursors read for the next range
+        __syncthreads();  // the list is rebuilt, the bitmaps are stored
+    }
+    const u32 n16 = (u32)(rows >> 7);
+    const uint4* b16 = reinterpret_cast<const uint4*>(bm);
+    uint4* out = reinterpret_cast<uint4*>(B + t * g.nw + (w0 << (g.wl - 6)));
+    for (u32 j = tid; j < n16; j += kWinThreads) out[j] = b16[j];
+    if (TWICE) {
+        const uint4* c16 = reinterpret_cast<const uint4*>(bm2);
+        uint4* out2 = reinterpret_cast<uint4*>(B2 + t * g.nw + (w0 << (g.wl - 6)));
+        for (u32 j = tid; j < n16; j += kWinThreads) out2[j] = c16[j];
     }
 }
 
@@ -188,63 +345,85 @@ k_win_tiles(const u64* __restrict__ ids, Plan plan, WinGeom g, u64* __restrict__
 // = rows of two or more tiles, class 1 + t = rows of tile t alone (with the
 // two-or-more filter: rows tile t holds twice or more and no other tile
 // holds); the class words, every word's rank within the window (the class's
-// rows below it, 16 bits: a window has at most 2^16 rows), and the window's
-// rows per class.  Thread i takes the window's words [kClassWords i,
-// kClassWords (i + 1)); the words are formed twice (for the counts, then for
-// the ranks), the second time from tile words still in L1.
-__global__ void __launch_bounds__(kClassThreads, 4)
+// rows of the window below the word, 16 bits: a window has at most 2^16
+// rows), and the window's rows per class.  Thread i takes the window's words
+// 2 i and 2 i + 1, every tile's in registers (up to MT tiles), so each is
+// read once; the counts of three classes share a 64-bit scan, and all scans
+// one pair of barriers.
+template <int MT>
+__global__ void __launch_bounds__(kClassThreads)
 k_win_classify(const u64* __restrict__ B, const u64* __restrict__ B2, WinGeom g, u64* __restrict__ cls,
                unsigned short* __restrict__ pre, u32* __restrict__ cnt)
 {
-    __shared__ u64 s_scan[kClassThreads / 32];
-    const int tid = threadIdx.x;
+    constexpr int kScans = (MT + 3) / 3;  // of MT + 1 classes, three a scan (fields of 21 bits)
+    __shared__ u64 s_scan[kScans][kClassThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const u64 w = blockIdx.x, W64 = 1ull << (g.wl - 6);
-    const u64 j0 = w * W64 + (u64)tid * kClassWords;
-    const bool mine = (u64)tid * kClassWords < W64;
-    u64 twos[kClassWords];
-    #pragma unroll
-    for (int i = 0; i < kClassWords; ++i) {
-        u64 ones = 0, tw = 0;
-        if (mine)
-            for (u64 q = 0; q < g.T; ++q) {
-                const u64 v = B[q * g.nw + j0 + i];
-                tw |= ones & v;
-                ones |= v;
-            }
-        twos[i] = tw;
+    const u64 j0 = w * W64 + 2 * (u64)tid;
+    const bool mine = 2 * (u64)tid < W64;
+    ulonglong2 c[MT + 1];
+    {
+        ulonglong2 ones = make_ulonglong2(0, 0), twos = ones;
+        #pragma unroll
+        for (int q = 0; q < MT; ++q) {
+            const ulonglong2 v = mine && q < (int)g.T ? *(const ulonglong2*)(B + q * g.nw + j0) : make_ulonglong2(0, 0);
+            twos.x |= ones.x & v.x;
+            twos.y |= ones.y & v.y;
+            ones.x |= v.x;
+            ones.y |= v.y;
+            c[q + 1] = v;
+        }
+        c[0] = twos;
+        #pragma unroll
+        for (int q = 0; q < MT; ++q) {
+            if (B2 && mine && q < (int)g.T) c[q + 1] = *(const ulonglong2*)(B2 + q * g.nw + j0);
+            c[q + 1].x &= ~twos.x;
+            c[q + 1].y &= ~twos.y;
+        }
     }
-    auto word = [&](u64 q, int i) -> u64 {  // class q's word i of this thread
-        if (q == 0) return twos[i];
-        const u64 v = B2 ? B2[(q - 1) * g.nw + j0 + i] : B[(q - 1) * g.nw + j0 + i];
-        return v & ~twos[i];
-    };
-    // counts of this thread's words, three classes to a scan (fields of 21 bits)
-    for (u64 q0 = 0; q0 <= g.T; q0 += 3) {
+    u64 own[kScans], inc[kScans];
+    #pragma unroll
+    for (int s = 0; s < kScans; ++s) {
         u64 packed = 0;
-        for (u64 f = 0; f < 3 && q0 + f <= g.T; ++f) {
-            u64 sum = 0;
-            if (mine)
-                #pragma unroll
-                for (int i = 0; i < kClassWords; ++i) {
-                    const u64 v = word(q0 + f, i);
-                    cls[(q0 + f) * g.nw + j0 + i] = v;
-                    sum += (u64)__popcll(v);
-                }
-            packed |= sum << (21 * f);
+        #pragma unroll
+        for (int f = 0; f < 3; ++f)
+            if (3 * s + f <= MT) packed |= (u64)(__popcll(c[3 * s + f].x) + __popcll(c[3 * s + f].y)) << (21 * f);
+        own[s] = packed;
+        u64 x = packed;
+        #pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const u64 y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
         }
-        u64 ex;
-        const u64 tot = block_exclusive_scan<kClassThreads>(packed, ex, s_scan);
-        for (u64 f = 0; f < 3 && q0 + f <= g.T; ++f) {
-            const u64 q = q0 + f;
-            u32 run = (u32)((ex >> (21 * f)) & 0x1fffffull);
-            if (mine)
-                #pragma unroll
-                for (int i = 0; i < kClassWords; ++i) {
-                    pre[q * g.nw + j0 + i] = (unsigned short)run;
-                    run += (u32)__popcll(cls[q * g.nw + j0 + i]);
-                }
-            if (tid == 0) cnt[q * g.nwin + w] = (u32)((tot >> (21 * f)) & 0x1fffffull);
+        inc[s] = x;
+        if (lane == 31) s_scan[s][warp] = x;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        #pragma unroll
+        for (int s = 0; s < kScans; ++s) {
+            u64 x = lane < kClassThreads / 32 ? s_scan[s][lane] : 0;
+            #pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const u64 y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            if (lane < kClassThreads / 32) s_scan[s][lane] = x;
         }
+    }
+    __syncthreads();
+    #pragma unroll
+    for (int q = 0; q <= MT; ++q) {
+        if (q > (int)g.T) break;
+        const int s = q / 3, sh = 21 * (q % 3);
+        const u64 ex = (warp ? s_scan[s][warp - 1] : 0) + inc[s] - own[s];
+        const u32 run = (u32)(ex >> sh) & 0x1fffffu;
+        if (mine) {
+            *(ulonglong2*)(cls + q * g.nw + j0) = c[q];
+            *(ushort2*)(pre + q * g.nw + j0) =
+                make_ushort2((unsigned short)run, (unsigned short)(run + (u32)__popcll(c[q].x)));
+        }
+        if (tid == 0) cnt[q * g.nwin + w] = (u32)(s_scan[s][kClassThreads / 32 - 1] >> sh) & 0x1fffffu;
     }
 }
 
@@ -252,9 +431,9 @@ k_win_classify(const u64* __restrict__ B, const u64* __restrict__ B2, WinGeom g,
 // range), and the rows of all classes into plan.totals.
 __global__ void k_win_agg(const u32* __restrict__ cnt, WinGeom g, Plan plan, u64* __restrict__ agg)
 {
-    const u64 i = blockIdx.x * (u64)blockDim.x + threadIdx.x;
+    const u32 i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (g.T + 1) * g.G) return;
-    const u64 c = i / g.G, r = i - c * g.G;
+    const u32 c = i / (u32)g.G, r = i - c * (u32)g.G;
     const u64 w0 = r * g.wpc, w1 = min(w0 + g.wpc, g.nwin);
     u64 s = 0;
     for (u64 w = w0; w < w1; ++w) s += cnt[c * g.nwin + w];
@@ -262,202 +441,204 @@ __global__ void k_win_agg(const u32* __restrict__ cnt, WinGeom g, Plan plan, u64
     if (s) atomicAdd((unsigned long long*)(plan.totals + kPlanRowsTotal), (unsigned long long)s);
 }
 
-// Pass 2 state of one class of a range: the rows' first word of the range
-// in the matrix (row kk of the tile at base + kk * stride) and the range's
-// words per row (a multiple-of-64 rank count / 64).
-struct RangeClass {
-    u64* base;
-    u64 stride;
-    u32 qn;
-};
-
-// Store the staged words [blk, blk + kStage) of the range and clear them.
-__device__ __forceinline__ void rc_flush(const RangeClass& c, u64* row, u32 blk, u64* st, int lane)
-{
-    __syncwarp();
-    #pragma unroll
-    for (int i = 0; i < kStage / 32; ++i) {
-        const u32 q = blk + (u32)(32 * i + lane);
-        if (q < c.qn) row[q] = st[32 * i + lane];
-        st[32 * i + lane] = 0ull;
-    }
-    __syncwarp();
-}
-
-// Put bit `bit` of word q (lanes with has) into the staged words from blk
-// on; the staged block moves forward as the sample's ranks pass it, and the
-// words it passes over are stored as zeros.  Ranks grow along a sample's
-// sorted values, so the lowest pending lane holds the lowest pending word;
-// a word outside the range (only from unsorted input) is dropped.
-__device__ __forceinline__ void rc_place(const RangeClass& c, u64* row, u32& blk, u64* st, bool has, u32 q, u64 bit,
-                                         int lane)
-{
-    for (;;) {
-        const bool fit = has && q >= blk && q < blk + kStage && q < c.qn;
-        if (fit) atomicOr((unsigned long long*)(st + (q - blk)), (unsigned long long)bit);
-        has = has && !fit && q >= blk && q < c.qn;
-        const unsigned pend = __ballot_sync(0xffffffffu, has);
-        if (!pend) return;
-        const u32 qmin = __shfl_sync(0xffffffffu, q, __ffs((int)pend) - 1);
-        rc_flush(c, row, blk, st, lane);
-        const u32 tgt = blk + (qmin - blk) / kStage * kStage;
-        for (u32 z = blk + kStage + (u32)lane; z < tgt; z += 32) row[z] = 0ull;
-        blk = tgt;
-    }
-}
-
 // Pass 2: CTA (range r, tile t) = blockIdx.x (r * T + t) packs the tile's
-// samples over the whole range.  Shared memory: the range's class-0 and
-// class-(1 + t) words, their ranks within each window, and the staged words
-// of every warp's sample.  A warp packs one sample at a time,
-// kDepth2 x 32 consecutive values per step; a sample's ranks run on from
-// window to window, and the range holds whole words, so every word is
-// stored once, by its sample's warp.
-__global__ void __launch_bounds__(kWin2Threads, 2)
-k_win_pack(const u64* __restrict__ ids, WinGeom g, const u64* __restrict__ cls,
+// samples over the range.  Shared memory: per class (0 and 1 + t) and 32 rows
+// the class bits and the rank of the first of them, then the gathered words,
+// then the list.  A value costs one or two of these lookups and one shared
+// OR.
+__global__ void __launch_bounds__(kWinThreads, 2)
+k_win_pack(Values v, WinGeom g, const u64* __restrict__ cls,
            const unsigned short* __restrict__ pre, const u32* __restrict__ cnt, const u64* __restrict__ boff,
            const u64* __restrict__ curs, const u64* __restrict__ kbase, u64* XM, u64 stride_m, u64* XS, u64 stride_s)
 {
     extern __shared__ __align__(16) unsigned char win_smem[];
-    const u32 W64 = (u32)(1u << (g.wl - 6));
-    const u64 r = blockIdx.x / g.T, t = blockIdx.x % g.T;
-    const u64 w0 = r * g.wpc, w1 = min(w0 + g.wpc, g.nwin);
-    const u32 nwr = (u32)(w1 - w0), RW = nwr * W64;  // the range's windows and words per class
-    u64* sW = reinterpret_cast<u64*>(win_smem);                                 // [2][RW]
-    u64* stage = sW + 2 * (u64)g.wpc * W64;                                     // [warps][2][kStage]
-    unsigned short* sP = reinterpret_cast<unsigned short*>(stage + kWin2Warps * 2 * kStage);  // [2][RW]
+    const u32 r = blockIdx.x / (u32)g.T, t = blockIdx.x - r * (u32)g.T;
+    const u64 w0 = (u64)r << g.wpc_log, w1 = min(w0 + g.wpc, g.nwin);
+    const u32 nwr = (u32)(w1 - w0), RW = nwr << (g.wl - 6);  // the range's windows and words per class
+    uint2* e0 = reinterpret_cast<uint2*>(win_smem);
+    uint2* e1 = e0 + (g.wpc << (g.wl - 5));
+    u64* stage = reinterpret_cast<u64*>(e1 + (g.wpc << (g.wl - 5)));
+    PieceList& L = *reinterpret_cast<PieceList*>(stage + kStageWords);
     __shared__ u32 s_wb[2][kMaxWinPerRange];
     __shared__ u64 s_rb[2];
-    __shared__ u32 s_qn[2];
-    __shared__ u32 s_next;
+    __shared__ u32 s_qn[2], s_inv, s_gs, s_rounds;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const u64 k0 = t * kWinTile, m = min(kWinTile, g.n - k0);
-    const u64 cl1 = 1 + t;
+    const u32 cl1 = 1 + t;
 
-    for (int i = tid; i < kWin2Warps * 2 * kStage; i += kWin2Threads) stage[i] = 0ull;
-    for (u32 j = tid; j < RW; j += kWin2Threads) {
-        sW[j] = cls[w0 * W64 + j];
-        sW[RW + j] = cls[cl1 * g.nw + w0 * W64 + j];
-        sP[j] = pre[w0 * W64 + j];
-        sP[RW + j] = pre[cl1 * g.nw + w0 * W64 + j];
-    }
-    if (tid == 0) s_next = 0;
     if (tid < 2) {
-        const u64 c = tid ? cl1 : 0;
+        const u32 c = tid ? cl1 : 0;
         u32 s = 0;
         for (u32 wi = 0; wi < nwr; ++wi) {
             s_wb[tid][wi] = s;
             s += cnt[c * g.nwin + w0 + wi];
         }
         s_rb[tid] = (boff[c * g.G + r] - boff[c * g.G]) / 64;  // ranges start on whole words
-        s_qn[tid] = (s + 63) / 64;
+        s_qn[tid] = (tid ? XS : XM) ? (s + 63) / 64 : 0;
+    }
+    if (tid < 32) {
+        __syncwarp();
+        if (tid == 0) {
+            const u32 l = max(s_qn[0] + s_qn[1], 1u);
+            s_rounds = 0;
+            // i / l by a multiplication (exact: i l < 2^32; l = 1 has no 32-bit reciprocal)
+            s_inv = l > 1 ? 0xffffffffu / l + 1 : 0;
+            s_gs = min((u32)m, kStageWords / l);  // samples gathered at a time (l <= 2 * 2048: at least one)
+        }
     }
     __syncthreads();
-
-    RangeClass cl[2];
-    cl[0].base = XM ? XM + k0 * stride_m + kbase[0] + s_rb[0] : nullptr;
-    cl[0].stride = stride_m;
-    cl[0].qn = XM ? s_qn[0] : 0;
-    cl[1].base = XS ? XS + k0 * stride_s + kbase[cl1] + s_rb[1] : nullptr;
-    cl[1].stride = stride_s;
-    cl[1].qn = XS ? s_qn[1] : 0;
-    u64* st_w = stage + warp * 2 * kStage;
-    const u64 rlo = g.lo + (w0 << g.wl), rows_r = (u64)nwr << g.wl;
-
-    // the tile's samples, one per warp at a time (they go to warps as the
-    // warps finish one): its segment of the range, up to 4 x 32 values per step
-    const int wsh = g.wl - 6;  // words of a window = 1 << wsh
-    for (;;) {
-        u32 e32 = 0;
-        if (lane == 0) {
-            e32 = atomicAdd(&s_next, 1u);
-            if (e32 < m) e32 = g.lpt[k0 + e32];  // largest samples first
+    const u32 q0 = s_qn[0], Lw = q0 + s_qn[1], inv = s_inv, gs = s_gs;
+    if (Lw == 0) return;
+    #pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        // two words a thread and step: their four half-words and ranks
+        const u64 at = (c ? cl1 * g.nw : 0) + (w0 << (g.wl - 6));
+        const ulonglong2* cw = reinterpret_cast<const ulonglong2*>(cls + at);
+        const ushort2* cp = reinterpret_cast<const ushort2*>(pre + at);
+        uint4* e = reinterpret_cast<uint4*>(c ? e1 : e0);
+        for (u32 j = tid; j < RW / 2; j += kWinThreads) {
+            const ulonglong2 w = cw[j];
+            const ushort2 p = cp[j];
+            const u32 wb = s_wb[c][j >> (g.wl - 7)], p0 = wb + p.x, p1 = wb + p.y;
+            e[2 * j] = make_uint4((u32)w.x, p0, (u32)(w.x >> 32), p0 + (u32)__popc((u32)w.x));
+            e[2 * j + 1] = make_uint4((u32)w.y, p1, (u32)(w.y >> 32), p1 + (u32)__popc((u32)w.y));
         }
-        const u64 e = __shfl_sync(0xffffffffu, e32, 0);
-        if (e >= m) break;
-        const u64 a = curs[r * g.n + k0 + e], b = max(a, curs[(r + 1) * g.n + k0 + e]);
-        u64* row0 = cl[0].base ? cl[0].base + e * cl[0].stride : nullptr;
-        u64* row1 = cl[1].base ? cl[1].base + e * cl[1].stride : nullptr;
-        u32 blk0 = 0, blk1 = 0;
-        for (u64 p = a; p < b; p += kDepth2 * 32) {
-            u64 x[kDepth2];
-            #pragma unroll
-            for (int i = 0; i < kDepth2; ++i) {
-                const u64 pos = p + (u64)(32 * i + lane);
-                x[i] = pos < b ? ids[pos] : 0ull;
-            }
-            #pragma unroll
-            for (int i = 0; i < kDepth2; ++i) {
-                if (p + (u64)(32 * i) >= b) break;
-                // class and rank of this lane's value: class 0 if its row is
-                // held by two or more tiles, else the tile's class if kept there
-                const u64 d64 = x[i] - rlo;
-                const bool in = p + (u64)(32 * i + lane) < b && d64 < rows_r;
-                const u32 d = in ? (u32)d64 : 0u, j = d >> 6, sh = d & 63u;
-                const u64 c0w = sW[j], c1w = sW[RW + j];
-                const bool h0 = in && ((c0w >> sh) & 1ull), h1 = in && !h0 && ((c1w >> sh) & 1ull);
-                const u32 cc = h1 ? 1u : 0u;
-                const u32 rk = s_wb[0][cc * kMaxWinPerRange + (j >> wsh)] + (u32)sP[cc * RW + j] +
-                               (u32)__popcll((h1 ? c1w : c0w) & ((1ull << sh) - 1ull));
-                const bool has = h0 || h1;
-                const u32 q = rk >> 6;
-                const u64 bit = 1ull << (rk & 63u);
-                const u32 bk = h1 ? blk1 : blk0, qn = h1 ? cl[1].qn : cl[0].qn;
-                const bool fit = has && q >= bk && q < bk + kStage && q < qn;
-                if (!__any_sync(0xffffffffu, has && !fit)) {
-                    if (fit) atomicOr((unsigned long long*)(st_w + cc * kStage + (q - bk)), (unsigned long long)bit);
-                } else {
-                    rc_place(cl[0], row0, blk0, st_w, h0, q, bit, lane);
-                    rc_place(cl[1], row1, blk1, st_w + kStage, h1, q, bit, lane);
+    }
+    u64 a = 0, b = 0;
+    if (tid < m) {
+        a = curs[r * g.n + k0 + tid];
+        b = max(a, curs[(r + 1) * g.n + k0 + tid]);
+        if (b > a) atomicMax(&s_rounds, (u32)((b - a + kRoundLen - 1) / kRoundLen));
+    }
+    // rows modulo the range (see pass 1): a row has a place only where its class bit is set
+    const u32 rlo32 = (u32)(g.lo + (w0 << g.wl)), mask = (nwr << g.wl) - 1;
+    u32* stage32 = reinterpret_cast<u32*>(stage);
+    __syncthreads();
+    const u32 rounds = s_rounds;
+    for (u32 g0 = 0; g0 < (u32)m; g0 += gs) {
+        const u32 g1 = min((u32)m, g0 + gs);
+        for (u32 i = tid; i < ((g1 - g0) * Lw + 1) / 2; i += kWinThreads)
+            reinterpret_cast<uint4*>(stage)[i] = make_uint4(0u, 0u, 0u, 0u);
+        for (u32 rd = 0; rd < rounds; ++rd) {
+            const bool mine = (u32)tid >= g0 && (u32)tid < g1;
+            const u32 F = list_build(L, v, a, mine ? b : a, rd);
+            const u32 cw = (F + kWinThreads - 1) / kWinThreads * 32;  // a warp's share: whole steps of a piece a lane
+            const u32 f1 = min(F, (warp + 1) * cw);
+            u32 f = warp * cw + lane;
+            if (f < f1) {
+                Walk wk;
+                wk.init(L, v, f);
+                wk.to(L, v, f);
+                u32 nx[kRun];  // the next piece's values, loaded ahead
+                load_piece(v, wk, nx);
+                while (f < f1) {
+                    u32 x[kRun];
+                    #pragma unroll
+                    for (u32 i = 0; i < kRun; ++i) x[i] = nx[i];
+                    rows_of(x, wk.lo, wk.hi, rlo32, mask);
+                    const u32 at = (wk.k - g0) * 2 * Lw;
+                    f += 32;
+                    if (f < f1) {
+                        wk.to(L, v, f);
+                        load_piece(v, wk, nx);
+                    }
+                    #pragma unroll
+                    for (u32 i = 0; i < kRun; ++i) {
+                        // class 0 if two or more tiles hold the row, else the tile's
+                        // class if the row is kept there
+                        const u32 d = x[i], bit = 1u << (d & 31);
+                        uint2 e = e0[d >> 5];
+                        u32 to = at;
+                        if (!(e.x & bit)) {
+                            e = e1[d >> 5];
+                            to += 2 * q0;
+                        }
+                        if (e.x & bit) {
+                            const u32 rk = e.y + (u32)__popc(e.x & (bit - 1));
+                            atomicOr(stage32 + to + (rk >> 5), 1u << (rk & 31));
+                        }
+                    }
                 }
             }
+            __syncthreads();  // the words are stored, or the list is rebuilt
         }
-        rc_flush(cl[0], row0, blk0, st_w, lane);
-        for (u32 z = blk0 + kStage + (u32)lane; z < cl[0].qn; z += 32) row0[z] = 0ull;
-        rc_flush(cl[1], row1, blk1, st_w + kStage, lane);
-        for (u32 z = blk1 + kStage + (u32)lane; z < cl[1].qn; z += 32) row1[z] = 0ull;
+        if (rounds == 0) __syncthreads();
+        u64* dm = XM + (k0 + g0) * stride_m + kbase[0] + s_rb[0];
+        u64* ds = XS + (k0 + g0) * stride_s + kbase[cl1] + s_rb[1];
+        for (u32 i = tid; i < (g1 - g0) * Lw; i += kWinThreads) {
+            const u32 y = Lw > 1 ? __umulhi(i, inv) : i, x = i - y * Lw;
+            u64* row = x < q0 ? dm + y * stride_m + x : ds + y * stride_s + (x - q0);
+            *row = stage[i];
+        }
+        __syncthreads();  // the gathered words are cleared for the next samples
     }
 }
 
-}  // namespace
-
 size_t win_tiles_smem(const WinGeom& g, bool twice)
 {
-    return (size_t)(twice ? 2 : 1) * ((size_t)g.wpc << (g.wl - 3)) + 2 * kWinTile * 8;
+    return (size_t)(twice ? 2 : 1) * ((size_t)g.gw << (g.wl - 3)) + sizeof(PieceList);
 }
 
 size_t win_pack_smem(const WinGeom& g)
 {
-    const size_t RW = (size_t)g.wpc << (g.wl - 6);
-    return 2 * RW * 8 + (size_t)kWin2Warps * 2 * kStage * 8 + 2 * RW * 2;
+    return 2 * ((size_t)g.wpc << (g.wl - 5)) * sizeof(uint2) + kStageWords * sizeof(u64) + sizeof(PieceList);
 }
 
-cudaError_t launch_win_classes(const u64* ids, Plan plan, const WinGeom& g, bool twice, u64* B, u64* B2, u64* cls,
-                               unsigned short* pre, u32* cnt, u64* agg, u64* curs, cudaStream_t st)
+}  // namespace
+
+WinGeom win_geom(u64 n, u64 T, u64 lo, u64 width, int wl, bool twice)
 {
-    if (g.G == 0) return cudaSuccess;
+    WinGeom g{};
+    g.n = n;
+    g.T = T;
+    g.lo = lo;
+    g.wl = wl;
+    g.nwin = width >> wl;
+    g.nw = width / 64;
+    g.wpc_log = 1;
+    g.wpc = 2;
+    g.G = (g.nwin + g.wpc - 1) / g.wpc;
+    g.gw = twice ? 4 : 8;
+    g.NG = (g.nwin + g.gw - 1) / g.gw;
+    return g;
+}
+
+namespace {
+Values values_of(const u64* ids, u64 N) { return Values{ids, N, (u32)((uintptr_t)ids / 8 % 4)}; }
+}  // namespace
+
+cudaError_t launch_win_classes(const u64* ids, u64 N, Plan plan, const WinGeom& g, bool twice, u64* B, u64* B2, u64* cls,
+                               unsigned short* pre, u32* cnt, u64* agg, u64* gcurs, u64* curs, cudaStream_t st)
+{
+    if (g.nwin == 0) return cudaSuccess;
+    const u64 searches = (g.NG + kCursChunk - 1) / kCursChunk * g.n;
+    k_win_cursors<<<(unsigned)((searches + 127) / 128), 128, 0, st>>>(ids, plan, g, gcurs);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     const size_t smem = win_tiles_smem(g, twice);
-    const unsigned grid = (unsigned)((g.G + kTileRanges - 1) / kTileRanges * g.T);
-    cudaError_t e;
+    const unsigned grid = (unsigned)(g.NG * g.T);
     if (twice) {
         e = cudaFuncSetAttribute(k_win_tiles<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        k_win_tiles<true><<<grid, kWin1Threads, smem, st>>>(ids, plan, g, B, B2, curs);
+        k_win_tiles<true><<<grid, kWinThreads, smem, st>>>(values_of(ids, N), g, gcurs, B, B2, curs);
     } else {
         e = cudaFuncSetAttribute(k_win_tiles<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        k_win_tiles<false><<<grid, kWin1Threads, smem, st>>>(ids, plan, g, B, nullptr, curs);
+        k_win_tiles<false><<<grid, kWinThreads, smem, st>>>(values_of(ids, N), g, gcurs, B, nullptr, curs);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_win_classify<<<(unsigned)g.nwin, kClassThreads, 0, st>>>(B, twice ? B2 : nullptr, g, cls, pre, cnt);
+    const u64* b2 = twice ? B2 : nullptr;
+    if (g.T <= 4) k_win_classify<4><<<(unsigned)g.nwin, kClassThreads, 0, st>>>(B, b2, g, cls, pre, cnt);
+    else if (g.T <= 8) k_win_classify<8><<<(unsigned)g.nwin, kClassThreads, 0, st>>>(B, b2, g, cls, pre, cnt);
+    else k_win_classify<16><<<(unsigned)g.nwin, kClassThreads, 0, st>>>(B, b2, g, cls, pre, cnt);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_win_agg<<<(unsigned)(((g.T + 1) * g.G + 255) / 256), 256, 0, st>>>(cnt, g, plan, agg);
     return cudaGetLastError();
 }
 
-cudaError_t launch_win_pack(const u64* ids, const WinGeom& g, const u64* cls, const unsigned short* pre,
+cudaError_t launch_win_pack(const u64* ids, u64 N, const WinGeom& g, const u64* cls, const unsigned short* pre,
                             const u32* cnt, const u64* boff, const u64* curs, const u64* kbase, u64* XM, u64 stride_m,
                             u64* XS, u64 stride_s, cudaStream_t st)
 {
@@ -465,8 +646,8 @@ cudaError_t launch_win_pack(const u64* ids, const WinGeom& g, const u64* cls, co
     const size_t smem = win_pack_smem(g);
     cudaError_t e = cudaFuncSetAttribute(k_win_pack, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_win_pack<<<(unsigned)(g.G * g.T), kWin2Threads, smem, st>>>(ids, g, cls, pre, cnt, boff, curs, kbase, XM,
-                                                                  stride_m, XS, stride_s);
+    k_win_pack<<<(unsigned)(g.G * g.T), kWinThreads, smem, st>>>(values_of(ids, N), g, cls, pre, cnt, boff, curs, kbase, XM,
+                                                                 stride_m, XS, stride_s);
     return cudaGetLastError();
 }
 
