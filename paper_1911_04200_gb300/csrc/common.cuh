@@ -186,12 +186,14 @@ struct TcJobDesc {
 // read by the kernels; with upload it is first written from `jobs`
 // (stream-ordered; not allowed while the stream is being captured).
 // tile_n: tiles of 128 x 256 (256) or 128 x 128 (128; a diagonal tile then
-// unpacks its rows once for both operands).  diag_only (tile_n 128, every job
-// of at most 128 samples: one diagonal tile each): stages of the A rows only,
-// more of them in flight.
+// unpacks its rows once for both operands).
 cudaError_t product_tc_jobs(const TcJobDesc* jobs, int njobs, void* dev_table, bool upload, int count_bits, int sms,
-                            u32* err, int timeout_ms, cudaStream_t st, int* launches, int tile_n = 256,
-                            bool diag_only = false);
+                            u32* err, int timeout_ms, cudaStream_t st, int* launches, int tile_n = 256);
+// Jobs of at most 128 samples each (W on the host), one diagonal 128 x 128
+// tile per job, up to 16 jobs a launch.  *taken false: a matrix's rows are not
+// 16-byte aligned, and nothing was launched.
+cudaError_t product_tc_diag(const TcJobDesc* jobs, int njobs, int count_bits, int sms, u32* err, int timeout_ms,
+                            cudaStream_t st, int* launches, bool* taken);
 bool product_tc_supported(int device);
 // Clock ticks of timeout_ms at the current device's maximum clock: the bound of
 // the tensor-core kernels' waits.  The clock is asked of the driver once per

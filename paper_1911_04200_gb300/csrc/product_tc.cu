@@ -71,13 +71,9 @@ constexpr u32 kErrTimeout = 4u;
 // The kernel's shape for tiles of 128 x TN (TN = 256 or 128).  One producer
 // thread per unpacked row (128 + TN), one MMA warp, four epilogue warps; two
 // TMEM accumulators of TN columns.  With TN = 128 a stage is two thirds the
-// size, so three stage buffers fit.  DG (TN = 128): every tile of the launch
-// is diagonal and a stage holds the A rows only - of SB = 512 bit-rows (four
-// atom columns, the two producer threads of a row writing two each), so the
-// per-stage costs are paid half as often; three buffers.
-template <int TN, bool DG = false, int SB = kStageBits>
+// size, so three stage buffers fit.
+template <int TN>
 struct Shape {
-    static constexpr int kN = TN;
     static constexpr int kRows = kM + TN;                  // rows unpacked per stage
     static constexpr int kProducerWarps = kRows / 32;
     static constexpr int kMmaWarp = kProducerWarps;
@@ -85,11 +81,8 @@ struct Shape {
     static constexpr int kWarps = kEpiWarp0 + 4;
     static constexpr int kThreads = kWarps * 32;
     static constexpr int kAtomB = TN * kBlkBytes;          // one atom column of B
-    static constexpr int kSB = SB;                         // bit-rows per stage
-    static constexpr int kSW = SB / 64;                    // packed words per stage
-    static constexpr int kAtomsS = SB / 128;               // atom columns per stage
-    static constexpr int kStageBytes = DG ? kAtomsS * kAtomA : kAtoms * kRows * kBlkBytes;
-    static constexpr int kBufs = DG ? 3 : TN == 128 ? 3 : 2;
+    static constexpr int kStageBytes = kAtoms * kRows * kBlkBytes;
+    static constexpr int kBufs = TN == 128 ? 3 : 2;
     static constexpr int kSmemBytes = kBufs * kStageBytes + 1024;  // + alignment slack
     static constexpr int kTmemCols = 2 * TN;               // two TN-column FP32 accumulators
     // instruction descriptor: kind::f8f6f4, D = F32, A = B = E4M3, both
@@ -100,8 +93,6 @@ struct Shape {
     static_assert(kEpiWarp0 % 4 == 1, "epilogue warp e reads TMEM lanes of warp rank (kEpiWarp0 + e) % 4");
     static_assert(kSmemBytes + 9 * 1024 <= 232448, "fits the per-CTA shared-memory limit");
     static_assert(TN == 128 || TN == 256, "tile widths");
-    static_assert(!DG || TN == kM, "diagonal-only launches have square tiles");
-    static_assert(SB == kStageBits || (DG && SB == 2 * kStageBits), "512-bit stages for diagonal-only launches");
 };
 
 __device__ __forceinline__ u32 smem_u32(const void* p) { return (u32)__cvta_generic_to_shared(p); }
@@ -185,14 +176,11 @@ struct TcJobs {
     int vec16;  // 16-byte loads are safe for every job
 };
 
-template <typename CT, int TN, bool DG, int SB>
-__global__ void __launch_bounds__(Shape<TN, DG, SB>::kThreads, 1)
+template <typename CT, int TN>
+__global__ void __launch_bounds__(Shape<TN>::kThreads, 1)
 k_prod_tc(const TcJobs P, u32* err, long long budget)
 {
-    using S = Shape<TN, DG, SB>;
-    constexpr int kSW = S::kSW;                    // packed words per stage
-    constexpr u64 kSeg = (1ull << 22) / SB;        // stages per segment under the exactness cap
-    constexpr bool kWide = SB == 2 * kStageBits;   // a diagonal row split into two halves of two atom columns
+    using S = Shape<TN>;
     constexpr int kBufs = S::kBufs, kStageBytes = S::kStageBytes, kAtomB = S::kAtomB;
     constexpr int kProducerWarps = S::kProducerWarps, kMmaWarp = S::kMmaWarp, kEpiWarp0 = S::kEpiWarp0;
     constexpr int kTmemCols = S::kTmemCols;
@@ -211,7 +199,7 @@ k_prod_tc(const TcJobs P, u32* err, long long budget)
         for (u32 j = 0; j < njobs; ++j) {
             const TcJob& J = P.job[j];
             const u64 W = J.Wdev ? *(volatile const u64*)J.Wdev : J.W;
-            const JobInfo x = tcs::job_info(J.n, W, U, TN, kSW);
+            const JobInfo x = tcs::job_info(J.n, W, U, TN);
             U += x.tiles * x.nst;
             ji[j] = x;
         }
@@ -268,7 +256,6 @@ k_prod_tc(const TcJobs P, u32* err, long long budget)
         // row and column), stage, and stages left in it
         WorkIter fit;
         fit.init(ji, njobs, gridDim.x, blockIdx.x);
-        fit.max_seg = kSeg;
         Seg fs;
         u64 f_key = ~0ull, f_kst = 0, f_left = 0, f_r0 = 0, f_c0 = 0, f_n = 0, f_W = 0, f_stride = 0;
         const u64* f_X = nullptr;
@@ -290,20 +277,18 @@ k_prod_tc(const TcJobs P, u32* err, long long budget)
                     f_key = key;
                 }
             }
-            dg = DG || (TN == kM && f_r0 == f_c0);
+            dg = TN == kM && f_r0 == f_c0;
             const u64 grow = tcs::fetch_row(p, f_r0, f_c0);  // on a diagonal tile both sides map to row f_r0 + row
             if (grow < f_n) {
                 const u64* src = f_X + grow * f_stride;
                 #pragma unroll
                 for (int q = 0; q < kStageWords; q += 2) {
-                    // the words of this thread's atom columns: with 256-bit
-                    // stages one column each on a diagonal tile, with 512-bit
-                    // stages the A side's first two and the B side's last two
-                    if (!kWide && dg && (q >> 1) != (is_a ? 0 : 1)) continue;
-                    const int qw = kWide ? q + (is_a ? 0 : kStageWords) : q;
+                    // the words of this thread's atom columns: one each on a
+                    // diagonal tile
+                    if (dg && (q >> 1) != (is_a ? 0 : 1)) continue;
                     u64 w0, w1;
-                    const bool in0 = tcs::fetch_word(f_kst, qw, f_W, w0, kSW);
-                    const bool in1 = tcs::fetch_word(f_kst, qw + 1, f_W, w1, kSW);
+                    const bool in0 = tcs::fetch_word(f_kst, q, f_W, w0);
+                    const bool in1 = tcs::fetch_word(f_kst, q + 1, f_W, w1);
                     if (P.vec16 && in1) {
                         // two words of the stage in one 16-byte load
                         asm volatile("ld.global.nc.v2.u64 {%0,%1}, [%2];\n"
@@ -335,13 +320,11 @@ k_prod_tc(const TcJobs P, u32* err, long long budget)
                 #pragma unroll
                 for (int at = 0; at < kAtoms; ++at) {
                     // a diagonal tile's rows go to the A operand only (the MMA
-                    // reads them for both): with 256-bit stages atom column 0
-                    // from the A-side thread and 1 from the B-side thread of
-                    // the row; with 512-bit stages columns 0-1 and 2-3
-                    if (!kWide && diag[a] && at != (is_a ? 0 : 1)) continue;
-                    const int ga = kWide ? at + (is_a ? 0 : kAtoms) : at;
+                    // reads them for both): atom column 0 from the A-side
+                    // thread and 1 from the B-side thread of the row
+                    if (diag[a] && at != (is_a ? 0 : 1)) continue;
                     unsigned char* rowp = sm + b * kStageBytes +
-                                          (diag[a] ? (u32)(row * kBlkBytes + ga * kAtomA) : row_off + at * atom_step);
+                                          (diag[a] ? (u32)(row * kBlkBytes + at * kAtomA) : row_off + at * atom_step);
                     #pragma unroll
                     for (int c = 0; c < 8; ++c) {
                         // bits 128 at + 16c .. +15 of the stage row -> 16 bytes
@@ -369,10 +352,8 @@ k_prod_tc(const TcJobs P, u32* err, long long budget)
         if (lane == 0) {
             WorkIter it;
             it.init(ji, njobs, gridDim.x, blockIdx.x);
-            it.max_seg = kSeg;
             Slots sl;
             sl.init();
-            sl.max_seg = kSeg;
             u64 t = 0;
             Seg sg;
             bool ok = true;
@@ -402,14 +383,14 @@ k_prod_tc(const TcJobs P, u32* err, long long budget)
                 // a diagonal tile (TN = 128, rows = columns) multiplies its A rows by themselves
                 u64 r0, c0;
                 tc_tile(sg.tile, ji[sg.job].TM, r0, c0, TN);
-                const bool dg = DG || (TN == kM && r0 == c0);
+                const bool dg = TN == kM && r0 == c0;
                 for (u64 q = 0; q < len; ++q, ++t) {
                     const int b = (int)(t % kBufs);
                     if (!mbar_wait(&full_bar[b], (u32)((t / kBufs) & 1), budget, abort_v)) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                     const u32 abase = base + b * kStageBytes, bbase = dg ? abase : abase + kABytes;
                     #pragma unroll
-                    for (int k = 0; k < SB / 32; ++k) {
+                    for (int k = 0; k < kStageBits / 32; ++k) {
                         // K step k: atom column k / 4, 32-byte slice k % 4
                         u64 da = sw128_desc(abase + (k >> 2) * kAtomA + (k & 3) * 32);
                         u64 db = sw128_desc(bbase + (k >> 2) * kAtomB + (k & 3) * 32);
@@ -473,10 +454,8 @@ k_prod_tc(const TcJobs P, u32* err, long long budget)
         };
         WorkIter it;
         it.init(ji, njobs, gridDim.x, blockIdx.x);
-        it.max_seg = kSeg;
         Slots sl;
         sl.init();
-        sl.max_seg = kSeg;
         Seg sg;
         bool ok = true;
         while (ok && it.next(sg)) {
@@ -518,29 +497,23 @@ k_prod_tc(const TcJobs P, u32* err, long long budget)
     }
 }
 
-template <typename CT, int TN, bool DG = false, int SB = kStageBits>
+template <typename CT, int TN>
 cudaError_t launch(const TcJobs& P, int sms, u32* err, int timeout_ms, cudaStream_t st)
 {
-    using S = Shape<TN, DG, SB>;
+    using S = Shape<TN>;
     cudaError_t e =
-        cudaFuncSetAttribute(k_prod_tc<CT, TN, DG, SB>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmemBytes);
+        cudaFuncSetAttribute(k_prod_tc<CT, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmemBytes);
     if (e != cudaSuccess) return e;
-    k_prod_tc<CT, TN, DG, SB><<<(unsigned)sms, S::kThreads, S::kSmemBytes, st>>>(P, err, wait_budget(timeout_ms));
+    k_prod_tc<CT, TN><<<(unsigned)sms, S::kThreads, S::kSmemBytes, st>>>(P, err, wait_budget(timeout_ms));
     return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t product_tc_jobs(const TcJobDesc* jobs, int njobs, void* dev_table, bool upload, int count_bits, int sms,
-                            u32* err, int timeout_ms, cudaStream_t st, int* launches, int tile_n, bool diag_only)
+                            u32* err, int timeout_ms, cudaStream_t st, int* launches, int tile_n)
 {
     if (tile_n != 128 && tile_n != 256) return cudaErrorInvalidValue;
-    if (diag_only) {
-        // one 128 x 128 tile per job, on the diagonal
-        if (tile_n != 128) return cudaErrorInvalidValue;
-        for (int q = 0; q < njobs; ++q)
-            if (jobs[q].n > (u64)kM) return cudaErrorInvalidValue;
-    }
     // the table of every job, copied once to device memory (dev_table holds
     // njobs entries of TcJob); one launch per group of kMaxJobs jobs
     static_assert(sizeof(TcJob) == sizeof(TcJobDesc), "table entry layout");
@@ -562,10 +535,7 @@ cudaError_t product_tc_jobs(const TcJobDesc* jobs, int njobs, void* dev_table, b
         P.job = (const TcJob*)dev_table + j0;
         P.njobs = (u32)std::min(kMaxJobs, njobs - j0);
         P.vec16 = vec16;
-        if (diag_only)
-            e = count_bits == 64 ? launch<u64, 128, true, 2 * kStageBits>(P, sms, err, timeout_ms, st)
-                                 : launch<u32, 128, true, 2 * kStageBits>(P, sms, err, timeout_ms, st);
-        else if (tile_n == 128)
+        if (tile_n == 128)
             e = count_bits == 64 ? launch<u64, 128>(P, sms, err, timeout_ms, st)
                                  : launch<u32, 128>(P, sms, err, timeout_ms, st);
         else

@@ -64,10 +64,9 @@
 // time-out the CTA raises the error word, waits (bounded) for the MMAs and
 // copies already issued, and both CTAs meet at a cluster barrier before TMEM
 // is freed and the CTAs exit.
-#include <atomic>
-#include <cuda.h>
 #include <algorithm>
-#include "common.cuh"
+#include <atomic>
+#include "tensor_map.cuh"
 
 namespace jsim {
 
@@ -297,10 +296,6 @@ __device__ __forceinline__ void pair_tile(u64 t, u64& r0, u64& c0)
     r0 = t * kTile;
     c0 = j * kTile;
 }
-
-using PFN_encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                               const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                               CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 // Work of a cluster: the words are cut into nst units of 1024 bit-rows and
 // these into chunks of L; chunk k's (tile, unit) pairs are laid out tile-major
@@ -742,38 +737,6 @@ k_prod_tc2(const __grid_constant__ CUtensorMap map, const u64* __restrict__ X, u
     }
 }
 
-// The driver's tensor-map encoder (null: not available).
-PFN_encode tensor_map_encoder()
-{
-    static std::atomic<void*> fn{nullptr};
-    void* p = fn.load(std::memory_order_acquire);
-    if (!p) {
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-            q != cudaDriverEntryPointSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        fn.store(p, std::memory_order_release);
-    }
-    return (PFN_encode)p;
-}
-
-// The tensor map of the packed matrix (n rows of W words, `stride` apart) in
-// boxes of 128 rows x 16 words with the 128-byte swizzle; false where the
-// rows are not 16-byte aligned (or the encoder refuses).
-bool packed_map(const ProductArgs& a, CUtensorMap* map)
-{
-    if ((uintptr_t)a.X % 16 != 0 || a.stride % 2 != 0 || a.W >= (1ull << 31) || a.stride * 8 >= (1ull << 40)) return false;
-    PFN_encode enc = tensor_map_encoder();
-    if (!enc) return false;
-    const cuuint64_t dims[2] = {a.W, a.n}, strides[1] = {a.stride * 8};
-    const cuuint32_t box[2] = {(cuuint32_t)kUnitWords, (cuuint32_t)kHalf}, estr[2] = {1, 1};
-    return enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, (void*)a.X, dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 template <typename CT, bool TMA>
 cudaError_t run(ProductArgs& a, const CUtensorMap& map, cudaStream_t st)
 {
@@ -824,7 +787,8 @@ cudaError_t run(ProductArgs& a, const CUtensorMap& map, cudaStream_t st)
 cudaError_t product_tc_pair(ProductArgs& a, cudaStream_t st)
 {
     CUtensorMap map{};
-    if (packed_map(a, &map)) return a.count_bits == 64 ? run<u64, true>(a, map, st) : run<u32, true>(a, map, st);
+    if (packed_map(&map, a.X, a.n, a.W, a.stride, kUnitWords, CU_TENSOR_MAP_SWIZZLE_128B))
+        return a.count_bits == 64 ? run<u64, true>(a, map, st) : run<u32, true>(a, map, st);
     return a.count_bits == 64 ? run<u64, false>(a, map, st) : run<u32, false>(a, map, st);
 }
 

@@ -616,9 +616,13 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
             int launches = 0;
             // every job is one diagonal 128 x 128 tile: its rows are unpacked
             // once for both operands
-            CK(product_tc_jobs(jobs.data(), (int)jobs.size(), jobtab.p, true, ctx->opt.count_bits, ctx->sms,
-                               ctx->d_err, ctx->opt.timeout_ms > 0 ? ctx->opt.timeout_ms : 2000, cs, &launches, 128,
-                               true));
+            const int to = ctx->opt.timeout_ms > 0 ? ctx->opt.timeout_ms : 2000;
+            bool taken = false;
+            CK(product_tc_diag(jobs.data(), (int)jobs.size(), ctx->opt.count_bits, ctx->sms, ctx->d_err, to, cs,
+                               &launches, &taken));
+            if (!taken)
+                CK(product_tc_jobs(jobs.data(), (int)jobs.size(), jobtab.p, true, ctx->opt.count_bits, ctx->sms,
+                                   ctx->d_err, to, cs, &launches, 128));
             ctx->stats.product_launches += launches;
             ctx->stats.launches += launches;
         }
