@@ -507,8 +507,11 @@ k_prod_tc2(const __grid_constant__ CUtensorMap map, const u64* __restrict__ X, u
                     }
                 }
                 if (TMA && hs + 1 == kUnitStages) {
+                    // the slot has been read: the fence orders these reads
+                    // before the async proxy's next write to it
+                    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(&lde_bar[y]);  // the slot has been read
+                    if (lane == 0) mbar_arrive(&lde_bar[y]);
                 }
                 if (ok && !first && !mbar_wait(&empty_bar[b], par, budget, abort_v)) ok = false;
                 ok = __all_sync(0xffffffffu, ok);  // tcgen05.st is warp-wide

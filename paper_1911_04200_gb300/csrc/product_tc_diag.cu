@@ -238,8 +238,13 @@ k_prod_diag(const __grid_constant__ DiagParams P, u32* err, long long budget)
             bool ok = mbar_wait(&ldf_bar[y], lpar, budget, abort_v);
             const ulonglong2 w0 = *(const ulonglong2*)(slots + y * kSlotBytes + src);
             const ulonglong2 w1 = *(const ulonglong2*)(slots + y * kSlotBytes + src + 8 * 64);
+            // The slot has been read: the fence orders these reads before the
+            // async proxy's next write to it.  Without it the release overtook
+            // reads still in flight, and stages mixed old and new words when
+            // copy CTAs shared the SM.
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive(&lde_bar[y]);  // the slot has been read
+            if (lane == 0) mbar_arrive(&lde_bar[y]);
             ok = ok && (t < kBufs || mbar_wait(&empty_bar[b], par, budget, abort_v));
             if (!__all_sync(0xffffffffu, ok)) break;
             unsigned char* st = sm + b * kStageBytes + dst;
