@@ -66,7 +66,7 @@ cudaError_t launch_feed_piece(const u64* hv, u64* dv, const u64* off, u64 n, con
 // Windowed ingest of the block-sparse path: the batch [lo, lo + nwin 2^wl)
 // of a plan over n samples in tile order (tiles of 128) is cut into nwin
 // windows of 2^wl rows.  Pass 1 runs one CTA per (group of gw windows, tile),
-// pass 2 one per (range of wpc windows, tile); the last group or range may be
+// pass 2 one per range of wpc windows; the last group or range may be
 // shorter.  A group is whole ranges.
 constexpr u64 kMaxWinPerRange = 2;
 struct WinGeom {

@@ -12,14 +12,20 @@
 // shared memory), no lane idles on a short segment, every load is one full
 // sector, and nothing is paid per sample but its two cursors.  What bounds
 // them (1024 clade samples, 1.3e9 values, 20 values a sample and window of
-// 2^16 rows): pass 1 instruction issue (62 % of slots) at 4.0 TB/s; pass 2
-// the shared-memory pipe (57 %) and the barriers between its phases, at 2.7
-// TB/s.  Measured on the whole call, ms: a warp per sample and range 5.9 +
-// 13.0 (passes 1 and 2); a flat list of single values 6.5 + 11.8; runs of
-// four values a lane, loaded word by word 5.0 + 12.2; aligned pieces in one
-// 32-byte load 3.9 + 9.9, with 1.4 for the cursors.  Ranges of 1, 2 and 4
-// windows in pass 2 take 10.6, 9.9 and 10.4; three CTAs an SM of pass 1 cost
-// more in registers than they hide (4.9).
+// 2^16 rows): pass 1 instruction issue and the values' latency (3.6 ms, 4.1
+// TB/s); pass 2 the shared-memory pipe (about 11 cycles of it per 32 values
+// and lookup) and the latency of its phases (7.9 ms, 3.3 TB/s), which the
+// next tile's loads beside this tile's stores shorten.  Measured on the whole
+// call, ms of passes 1 and 2: a warp per sample and range 5.9 + 13.0; a flat
+// list of single values 6.5 + 11.8; runs of four values a lane, loaded word
+// by word 5.0 + 12.2; aligned pieces in one 32-byte load 3.9 + 9.9 (one CTA
+// per range and tile in pass 2); cheaper list entries and one CTA per range,
+// its class-0 words placed once for all tiles 3.6 + 9.0; loads beside the
+// stores, nothing spilled 3.6 + 7.9 (64 bytes of spills in that loop cost 1.8
+// ms: a spilled load waits for its value).  The cursors take 1.4.  Also
+// tried in pass 2: ranges of 1 and 4 windows 10.6 and 10.4 against 9.9 (2);
+// three pieces a lane in flight 10.2 against 9.9; L2 prefetch of the next
+// tile's values 8.5 against 7.9.
 //
 // k_win_cursors: every sample's position at each group of windows.  Pass 1
 // (k_win_tiles, one CTA per group and tile): the tile's filter bitmap of the
@@ -36,8 +42,8 @@
 // are zero rows of the packed matrix, which add nothing to C (Eq. 4) - so
 // that every packed word belongs to one range.
 //
-// Pass 2 (k_win_pack, one CTA per range and tile): the tile's samples are
-// packed into the class-0 matrix XM and the tile's matrix XS.  A value's
+// Pass 2 (k_win_pack, one CTA per range, tile after tile): the tile's samples
+// are packed into the class-0 matrix XM and the tile's matrix XS.  A value's
 // class and rank come from the range's class words and ranks in shared
 // memory; the words of a group of samples (as many as fit, usually the whole
 // tile) are gathered there too and stored whole with plain stores.  Every
@@ -51,10 +57,11 @@ namespace jsim {
 namespace {
 
 constexpr int kWinThreads = 512;
-constexpr u32 kRun = 4;           // values a lane takes at a time: 32 aligned bytes
+constexpr u32 kRun = 4;           // values of a piece: 32 aligned bytes
 constexpr int kClassThreads = 512;
 constexpr int kCursChunk = 8;     // consecutive cursors a thread of k_win_cursors finds
 constexpr u64 kWinTile = 128;     // samples per tile
+constexpr int kMaxClasses = 17;   // class 0 and up to 16 tiles'
 constexpr u32 kRoundLen = 1u << 24;     // values of a segment listed at a time (128 of them fit 32-bit positions)
 constexpr u32 kStageWords = 5120;       // words gathered at a time in pass 2 (40 KiB)
 
@@ -68,100 +75,110 @@ struct Values {
 
 // The flat list of up to 128 segments [a, b) of ids, in pieces (a segment's
 // first and last piece may hold other values too): segment k's pieces are
-// list entries [start[k], start[k + 1]).
+// list entries [beg, end).
+struct Segment {
+    u32 beg, end;
+    u32 words;  // list entry f of the segment holds values up to word words - 4 f of its piece
+    u32 skip;   // words of other values in its first piece
+};
 struct PieceList {
-    u64 a[kWinTile], b[kWinTile];
-    u32 start[kWinTile + 1];
+    Segment seg[kWinTile];
+    const u64* ptr[kWinTile];  // list entry f is the 32 bytes at ptr + 4 f
+    u64 a[kWinTile];
     u32 scan[kWinTile / 32];
 };
 
-// Lists values [r kRoundLen, (r + 1) kRoundLen) of every segment whose thread
-// (0 .. 127) has a < b; returns the list's length.  All threads call; the
-// list may be read after it, and rebuilt after a barrier.
-__device__ __forceinline__ u32 list_build(PieceList& L, const Values& v, u64 a, u64 b, u32 r)
+// Listing, in two parts around a barrier: values [r kRoundLen, (r + 1)
+// kRoundLen) of every segment whose thread (0 .. 127) has a < b.  count
+// returns what place needs; place returns the list's length.  The list may be
+// read after a barrier that follows, and rebuilt after another.
+struct Listing {
+    u64 a;
+    u32 len, runs, inc;
+};
+__device__ __forceinline__ Listing list_count(PieceList& L, const Values& v, u64 a, u64 b, u32 r)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    u32 runs = 0, inc = 0;
+    Listing x{0, 0, 0, 0};
     if (tid < (int)kWinTile) {
-        a = min(b, a + (u64)r * kRoundLen);
-        b = min(b, a + kRoundLen);
-        runs = a < b ? (u32)(((b - 1 + v.ph) >> 2) - ((a + v.ph) >> 2)) + 1 : 0;
-        inc = runs;
+        x.a = min(b, a + (u64)r * kRoundLen);
+        x.len = (u32)min(b - x.a, (u64)kRoundLen);
+        x.runs = x.len ? (u32)(((x.a + x.len - 1 + v.ph) >> 2) - ((x.a + v.ph) >> 2)) + 1 : 0;
+        x.inc = x.runs;
         #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const u32 y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += y;
+            const u32 y = __shfl_up_sync(0xffffffffu, x.inc, o);
+            if (lane >= o) x.inc += y;
         }
-        if (lane == 31) L.scan[warp] = inc;
-        L.a[tid] = a;
-        L.b[tid] = b;
+        if (lane == 31) L.scan[warp] = x.inc;
     }
-    __syncthreads();
+    return x;
+}
+__device__ __forceinline__ u32 list_place(PieceList& L, const Values& v, const Listing& x)
+{
+    const int tid = threadIdx.x, warp = tid >> 5;
     u32 total = 0, before = 0;
     #pragma unroll
     for (int w = 0; w < (int)kWinTile / 32; ++w) {
         if (w < warp) before += L.scan[w];
         total += L.scan[w];
     }
-    if (tid < (int)kWinTile) L.start[tid] = before + inc - runs;
-    if (tid == 0) L.start[kWinTile] = total;
-    __syncthreads();
+    if (tid < (int)kWinTile) {
+        const u32 beg = before + x.inc - x.runs, skip = (u32)(x.a + v.ph) & 3u;
+        L.seg[tid] = Segment{beg, beg + x.runs, 4 * beg + skip + x.len, skip};
+        L.ptr[tid] = v.ids + ((long long)((x.a + v.ph) >> 2) * 4 - (long long)v.ph - 4ll * beg);
+        L.a[tid] = x.a;
+    }
     return total;
 }
 
-// A lane's walk through a list, forward: its piece's segment k, the value
-// index of its first word (negative for a piece that begins before ids) and
-// the words [lo, hi) of it that belong to the segment.
+// A lane's walk through a list, forward: its segment k, its piece's address
+// and the words [lo, hi) of the piece that belong to the segment.
 struct Walk {
-    u32 k, beg, end, b, skip;  // segment; its list positions; low word of its end; words before it in its first piece
-    long long off;             // the segment's piece at list position f is off + f
-    long long base;
-    u32 lo, hi;
-    __device__ __forceinline__ void load(const PieceList& L, const Values& v)
-    {
-        beg = L.start[k];
-        end = L.start[k + 1];
-        const u64 sa = L.a[k] + v.ph;
-        skip = (u32)sa & 3u;
-        off = (long long)(sa >> 2) - (long long)beg;
-        b = (u32)L.b[k];
-    }
+    u32 k, lo, hi;
+    Segment sg;
+    const u64* ptr;
+    const u64* at;
     // at list position f (below the list's length)
-    __device__ __forceinline__ void init(const PieceList& L, const Values& v, u32 f)
+    __device__ __forceinline__ void init(const PieceList& L, u32 f)
     {
         u32 l = 0, h = kWinTile - 1;
         while (l < h) {
             const u32 mid = (l + h + 1) >> 1;
-            if (L.start[mid] <= f) l = mid; else h = mid - 1;
+            if (L.seg[mid].beg <= f) l = mid; else h = mid - 1;
         }
         k = l;
-        load(L, v);
+        sg = L.seg[k];
+        ptr = L.ptr[k];
     }
-    __device__ __forceinline__ void to(const PieceList& L, const Values& v, u32 f)
+    __device__ __forceinline__ void to(const PieceList& L, u32 f)
     {
-        if (f >= end) {
-            do ++k; while (f >= L.start[k + 1]);
-            load(L, v);
+        if (f >= sg.end) {
+            do {
+                ++k;
+                sg = L.seg[k];
+            } while (f >= sg.end);
+            ptr = L.ptr[k];
         }
-        base = 4 * (off + f) - (long long)v.ph;
-        lo = f == beg ? skip : 0;
-        hi = min(kRun, b - (u32)base);
+        at = ptr + 4ull * f;
+        lo = f == sg.beg ? sg.skip : 0;
+        hi = min(kRun, sg.words - 4 * f);
     }
 };
 
-// The low words of a piece's four values (a piece at either end of ids is
-// read value by value).
-__device__ __forceinline__ void load_piece(const Values& v, const Walk& w, u32 (&x)[kRun])
+// The low words of a piece's four values (with edge, where a list may reach
+// either end of ids, a piece that does is read value by value).
+__device__ __forceinline__ void load_piece(const Values& v, const Walk& w, bool edge, u32 (&x)[kRun])
 {
-    if (w.base >= 0 && w.base + (long long)kRun <= (long long)v.n) {
+    if (!edge || (w.at >= v.ids && w.at + kRun <= v.ids + v.n)) {
         u64 y[kRun];
         asm volatile("ld.global.nc.v4.u64 {%0,%1,%2,%3}, [%4];\n"
-                     : "=l"(y[0]), "=l"(y[1]), "=l"(y[2]), "=l"(y[3]) : "l"(v.ids + w.base));
+                     : "=l"(y[0]), "=l"(y[1]), "=l"(y[2]), "=l"(y[3]) : "l"(w.at));
         #pragma unroll
         for (u32 i = 0; i < kRun; ++i) x[i] = (u32)y[i];
     } else {
         #pragma unroll
-        for (u32 i = 0; i < kRun; ++i) x[i] = i >= w.lo && i < w.hi ? (u32)v.ids[w.base + i] : 0u;
+        for (u32 i = 0; i < kRun; ++i) x[i] = i >= w.lo && i < w.hi ? (u32)w.at[i] : 0u;
     }
 }
 
@@ -176,6 +193,9 @@ __device__ __forceinline__ void rows_of(u32 (&x)[kRun], u32 lo, u32 hi, u32 orig
     #pragma unroll
     for (u32 i = 1; i < kRun; ++i) x[i] = i >= hi ? x[i - 1] : x[i];
 }
+
+// Does the segment [a, b) reach a first or last piece of ids?
+__device__ __forceinline__ bool at_edge(const Values& v, u64 a, u64 b) { return a < b && (a < kRun || b + kRun > v.n); }
 
 // Every sample's position at the start of each group of g.gw windows (and at
 // the batch end): gcurs[g n + k] for entry k of the plan.  A thread bisects
@@ -235,7 +255,6 @@ k_win_tiles(Values v, WinGeom g, const u64* __restrict__ gcurs, u64* __restrict_
     u32* bm = reinterpret_cast<u32*>(win_smem);
     u32* bm2 = bm + (g.gw << (g.wl - 5));
     PieceList& L = *reinterpret_cast<PieceList*>(bm + (TWICE ? 2 : 1) * (g.gw << (g.wl - 5)));
-    __shared__ u32 s_rounds;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const u64 k0 = t * kWinTile, m = min(kWinTile, g.n - k0);
     // pass-2 ranges of the group: r0 on; a row of the group >> rsh is its range
@@ -243,92 +262,89 @@ k_win_tiles(Values v, WinGeom g, const u64* __restrict__ gcurs, u64* __restrict_
     const u32 nr = (u32)((w1 - w0 + g.wpc - 1) >> g.wpc_log);
     const int rsh = g.wl + g.wpc_log;
 
+    // everything the group needs first, in flight together
+    u64 a = 0, b = 0;
+    if (tid < m) {
+        a = gcurs[gi * g.n + k0 + tid];
+        b = max(a, gcurs[(gi + 1) * g.n + k0 + tid]);
+    }
     {
         uint4* z = reinterpret_cast<uint4*>(bm);
         const u32 nz = (u32)((TWICE ? 2 : 1) * (g.gw << (g.wl - 5)) / 4);
         for (u32 i = tid; i < nz; i += kWinThreads) z[i] = make_uint4(0u, 0u, 0u, 0u);
     }
-    if (tid == 0) s_rounds = 0;
-    __syncthreads();
-    u64 a = 0, b = 0;
     if (tid < m) {
-        a = gcurs[gi * g.n + k0 + tid];
-        b = max(a, gcurs[(gi + 1) * g.n + k0 + tid]);
         // the ranges no value crosses into start at the segment's end
         curs[r0 * g.n + k0 + tid] = a;
         for (u32 r = 1; r < nr; ++r) curs[(r0 + r) * g.n + k0 + tid] = b;
         if (w1 == g.nwin) curs[g.G * g.n + k0 + tid] = b;
-        if (b > a) atomicMax(&s_rounds, (u32)((b - a + kRoundLen - 1) / kRoundLen));
     }
-    __syncthreads();
-    const u32 rounds = s_rounds;
     // Rows are taken modulo the bitmap: a row outside the group only comes
     // from unsorted input, whose results are dropped.
     const u32 mask = (u32)(g.gw << g.wl) - 1;
-    for (u32 rd = 0; rd < rounds; ++rd) {
-        const u32 F = list_build(L, v, a, b, rd);
+    auto walk = [&](bool edge, u32 F, u32 rd) {
         const u32 cw = (F + kWinThreads - 1) / kWinThreads * 32;  // a warp's share: whole steps of a piece a lane
         const u32 f0 = warp * cw, f1 = min(F, f0 + cw);
-        if (f0 < f1) {
-            Walk wk;
-            wk.init(L, v, min(f0 + lane, f1 - 1));
-            u32 nx[kRun];  // the next piece's values, loaded ahead
-            wk.to(L, v, min(f0 + lane, f1 - 1));
-            load_piece(v, wk, nx);
-            u32 cd = 0;    // the row before the step's first piece
-            if (lane == 0 && (f0 != wk.beg || rd > 0)) cd = ((u32)v.ids[wk.base + wk.lo - 1] - glo32) & mask;
-            for (u32 f = f0 + lane; f - lane < f1; f += 32) {
-                u32 x[kRun];
-                #pragma unroll
-                for (u32 i = 0; i < kRun; ++i) x[i] = nx[i];
-                rows_of(x, wk.lo, wk.hi, glo32, mask);
-                const u32 k = wk.k;
-                const u64 s = (u64)wk.base;
-                const u32 lo = wk.lo;
-                const bool in = f < f1;
-                // the row before the piece, if it is of the sample's segment of the
-                // group (else 0: the first range's start)
-                const bool first = f == wk.beg;
-                u32 pd = __shfl_up_sync(0xffffffffu, x[kRun - 1], 1);
-                if (lane == 0) pd = cd;
-                cd = __shfl_sync(0xffffffffu, x[kRun - 1], 31);
-                bool prev = !first;
-                if (first) {
-                    pd = 0;
-                    if (rd > 0) {  // the list begins inside the segment
-                        pd = ((u32)v.ids[s + lo - 1] - glo32) & mask;
-                        prev = true;
-                    }
-                }
-                if (f + 32 < f1) {
-                    wk.to(L, v, f + 32);
-                    load_piece(v, wk, nx);
-                }
-                if (!in) continue;
-                if ((x[kRun - 1] >> rsh) > (pd >> rsh)) {
-                    // the values cross into further ranges
-                    u32 pr = pd >> rsh;
-                    #pragma unroll
-                    for (u32 i = 0; i < kRun; ++i) {
-                        const u32 rg = min(x[i] >> rsh, nr - 1);
-                        for (; pr < rg; ++pr) curs[(r0 + pr + 1) * g.n + k0 + k] = s + max(i, lo);
-                    }
-                }
+        if (f0 >= f1) return;
+        Walk wk;
+        wk.init(L, min(f0 + lane, f1 - 1));
+        wk.to(L, min(f0 + lane, f1 - 1));
+        u32 nx[kRun];  // the next piece's values, loaded ahead
+        load_piece(v, wk, edge, nx);
+        u32 cd = 0;    // the row before the step's first piece
+        if (lane == 0 && f0 != wk.sg.beg) cd = ((u32)wk.at[-1] - glo32) & mask;
+        for (u32 f = f0 + lane; f - lane < f1; f += 32) {
+            u32 x[kRun];
+            #pragma unroll
+            for (u32 i = 0; i < kRun; ++i) x[i] = nx[i];
+            rows_of(x, wk.lo, wk.hi, glo32, mask);
+            const u32 k = wk.k, lo = wk.lo;
+            const u64* at = wk.at;
+            const bool in = f < f1, first = f == wk.sg.beg;
+            // the row before the piece, if it is of the sample's segment of the
+            // group (else 0: the first range's start)
+            u32 pd = __shfl_up_sync(0xffffffffu, x[kRun - 1], 1);
+            if (lane == 0) pd = cd;
+            cd = __shfl_sync(0xffffffffu, x[kRun - 1], 31);
+            if (first) pd = rd > 0 ? ((u32)at[(int)lo - 1] - glo32) & mask : 0u;  // rd > 0: the list begins inside the segment
+            const bool prev = !first || rd > 0;
+            if (f + 32 < f1) {
+                wk.to(L, f + 32);
+                load_piece(v, wk, edge, nx);
+            }
+            if (!in) continue;
+            if ((x[kRun - 1] >> rsh) > (pd >> rsh)) {
+                // the values cross into further ranges
+                const u64 s = (u64)(at - v.ids);
+                u32 pr = pd >> rsh;
                 #pragma unroll
                 for (u32 i = 0; i < kRun; ++i) {
-                    const u32 bit = 1u << (x[i] & 31);
-                    if (TWICE) {
-                        if (i ? x[i] != x[i - 1] : !prev || x[0] != pd) {
-                            const u32 old = atomicOr(bm + (x[i] >> 5), bit);
-                            if (old & bit) atomicOr(bm2 + (x[i] >> 5), bit);
-                        }
-                    } else {
-                        atomicOr(bm + (x[i] >> 5), bit);
+                    const u32 rg = min(x[i] >> rsh, nr - 1);
+                    for (; pr < rg; ++pr) curs[(r0 + pr + 1) * g.n + k0 + k] = s + max(i, lo);
+                }
+            }
+            #pragma unroll
+            for (u32 i = 0; i < kRun; ++i) {
+                const u32 d = x[i], bit = 1u << (d & 31);
+                if (TWICE) {
+                    if (i ? d != x[i - 1] : !prev || d != pd) {
+                        const u32 old = atomicOr(bm + (d >> 5), bit);
+                        if (old & bit) atomicOr(bm2 + (d >> 5), bit);
                     }
+                } else {
+                    atomicOr(bm + (d >> 5), bit);
                 }
             }
         }
+    };
+    for (u32 rd = 0;; ++rd) {
+        const Listing x = list_count(L, v, a, b, rd);
+        const bool edge = __syncthreads_or(at_edge(v, a, b));
+        const u32 F = list_place(L, v, x);
+        const int more = __syncthreads_or(b - a > (u64)(rd + 1) * kRoundLen);  // segments beyond this round
+        walk(edge, F, rd);
         __syncthreads();  // the list is rebuilt, the bitmaps are stored
+        if (!more) break;
     }
     const u32 n16 = (u32)(rows >> 7);
     const uint4* b16 = reinterpret_cast<const uint4*>(bm);
@@ -441,136 +457,177 @@ __global__ void k_win_agg(const u32* __restrict__ cnt, WinGeom g, Plan plan, u64
     if (s) atomicAdd((unsigned long long*)(plan.totals + kPlanRowsTotal), (unsigned long long)s);
 }
 
-// Pass 2: CTA (range r, tile t) = blockIdx.x (r * T + t) packs the tile's
-// samples over the range.  Shared memory: per class (0 and 1 + t) and 32 rows
-// the class bits and the rank of the first of them, then the gathered words,
-// then the list.  A value costs one or two of these lookups and one shared
-// OR.
+// Pass 2: CTA r = blockIdx.x packs range r, tile after tile.  Shared memory:
+// per class (0, and 1 + t of the tile at hand) and 32 rows the class bits and
+// the place of the first of them among a sample's gathered bits, then the
+// gathered words, then the list.  A value costs one or two of these lookups
+// and one shared OR.  A tile's class words, ranks and cursors are loaded
+// while the words of the tile before are stored.
 __global__ void __launch_bounds__(kWinThreads, 2)
 k_win_pack(Values v, WinGeom g, const u64* __restrict__ cls,
            const unsigned short* __restrict__ pre, const u32* __restrict__ cnt, const u64* __restrict__ boff,
            const u64* __restrict__ curs, const u64* __restrict__ kbase, u64* XM, u64 stride_m, u64* XS, u64 stride_s)
 {
     extern __shared__ __align__(16) unsigned char win_smem[];
-    const u32 r = blockIdx.x / (u32)g.T, t = blockIdx.x - r * (u32)g.T;
+    const u32 r = blockIdx.x, T = (u32)g.T;
     const u64 w0 = (u64)r << g.wpc_log, w1 = min(w0 + g.wpc, g.nwin);
     const u32 nwr = (u32)(w1 - w0), RW = nwr << (g.wl - 6);  // the range's windows and words per class
     uint2* e0 = reinterpret_cast<uint2*>(win_smem);
     uint2* e1 = e0 + (g.wpc << (g.wl - 5));
     u64* stage = reinterpret_cast<u64*>(e1 + (g.wpc << (g.wl - 5)));
+    u32* stage32 = reinterpret_cast<u32*>(stage);
     PieceList& L = *reinterpret_cast<PieceList*>(stage + kStageWords);
-    __shared__ u32 s_wb[2][kMaxWinPerRange];
-    __shared__ u64 s_rb[2];
-    __shared__ u32 s_qn[2], s_inv, s_gs, s_rounds;
+    // per class: rows of the range's windows; the range's first word in the class's matrix
+    __shared__ u32 s_cnt[kMaxClasses][kMaxWinPerRange];
+    __shared__ u64 s_at[kMaxClasses];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const u64 k0 = t * kWinTile, m = min(kWinTile, g.n - k0);
-    const u32 cl1 = 1 + t;
+    const int wsh = g.wl - 6;  // words of a window = 1 << wsh
 
-    if (tid < 2) {
-        const u32 c = tid ? cl1 : 0;
-        u32 s = 0;
-        for (u32 wi = 0; wi < nwr; ++wi) {
-            s_wb[tid][wi] = s;
-            s += cnt[c * g.nwin + w0 + wi];
+    // words and ranks of class c: kWords words a thread, in flight together
+    constexpr u32 kWords = 4;  // (a range of 2^17 rows has 2048)
+    u64 cw[kWords];
+    u32 cp[kWords];
+    auto load_class = [&](u32 c) {
+        const u64* w = cls + (c * g.nw + (w0 << wsh));
+        const unsigned short* q = pre + (c * g.nw + (w0 << wsh));
+        #pragma unroll
+        for (u32 i = 0; i < kWords; ++i) {
+            const u32 j = tid + i * kWinThreads;
+            if (j < RW) {
+                cw[i] = w[j];
+                cp[i] = q[j];
+            }
         }
-        s_rb[tid] = (boff[c * g.G + r] - boff[c * g.G]) / 64;  // ranges start on whole words
-        s_qn[tid] = (tid ? XS : XM) ? (s + 63) / 64 : 0;
-    }
-    if (tid < 32) {
-        __syncwarp();
-        if (tid == 0) {
-            const u32 l = max(s_qn[0] + s_qn[1], 1u);
-            s_rounds = 0;
-            // i / l by a multiplication (exact: i l < 2^32; l = 1 has no 32-bit reciprocal)
-            s_inv = l > 1 ? 0xffffffffu / l + 1 : 0;
-            s_gs = min((u32)m, kStageWords / l);  // samples gathered at a time (l <= 2 * 2048: at least one)
+    };
+    // .. into e, the class's bits placed from bit `base` of a sample's gathered words
+    auto place_class = [&](uint2* e, u32 c, bool any, u32 base) {
+        #pragma unroll
+        for (u32 i = 0; i < kWords; ++i) {
+            const u32 j = tid + i * kWinThreads;
+            if (j < RW) {
+                const u64 w = any ? cw[i] : 0;
+                const u32 p = base + (j >> wsh ? s_cnt[c][0] : 0) + cp[i];
+                reinterpret_cast<uint4*>(e)[j] = make_uint4((u32)w, p, (u32)(w >> 32), p + (u32)__popc((u32)w));
+            }
         }
+    };
+    u64 a = 0, b = 0;  // (b is raised to a where they are used: unsorted input)
+    auto load_cursors = [&](u32 t) {
+        a = b = 0;
+        if (tid < (int)kWinTile && t * kWinTile + tid < g.n) {
+            a = curs[r * g.n + t * kWinTile + tid];
+            b = curs[(r + 1) * g.n + t * kWinTile + tid];
+        }
+    };
+    load_class(0);
+    if (tid < (int)(T + 1)) {
+        #pragma unroll
+        for (u32 w = 0; w < kMaxWinPerRange; ++w) s_cnt[tid][w] = w < nwr ? cnt[tid * g.nwin + w0 + w] : 0;
+        s_at[tid] = kbase[tid] + (boff[tid * g.G + r] - boff[tid * g.G]) / 64;  // ranges start on whole words
     }
+    load_cursors(0);
     __syncthreads();
-    const u32 q0 = s_qn[0], Lw = q0 + s_qn[1], inv = s_inv, gs = s_gs;
-    if (Lw == 0) return;
-    #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-        // two words a thread and step: their four half-words and ranks
-        const u64 at = (c ? cl1 * g.nw : 0) + (w0 << (g.wl - 6));
-        const ulonglong2* cw = reinterpret_cast<const ulonglong2*>(cls + at);
-        const ushort2* cp = reinterpret_cast<const ushort2*>(pre + at);
-        uint4* e = reinterpret_cast<uint4*>(c ? e1 : e0);
-        for (u32 j = tid; j < RW / 2; j += kWinThreads) {
-            const ulonglong2 w = cw[j];
-            const ushort2 p = cp[j];
-            const u32 wb = s_wb[c][j >> (g.wl - 7)], p0 = wb + p.x, p1 = wb + p.y;
-            e[2 * j] = make_uint4((u32)w.x, p0, (u32)(w.x >> 32), p0 + (u32)__popc((u32)w.x));
-            e[2 * j + 1] = make_uint4((u32)w.y, p1, (u32)(w.y >> 32), p1 + (u32)__popc((u32)w.y));
-        }
-    }
-    u64 a = 0, b = 0;
-    if (tid < m) {
-        a = curs[r * g.n + k0 + tid];
-        b = max(a, curs[(r + 1) * g.n + k0 + tid]);
-        if (b > a) atomicMax(&s_rounds, (u32)((b - a + kRoundLen - 1) / kRoundLen));
-    }
+    auto words_of = [&](u32 c) { return (s_cnt[c][0] + s_cnt[c][1] + 63) / 64; };
+    const u32 q0 = XM ? words_of(0) : 0;
+    place_class(e0, 0, q0 > 0, 0);
+    load_class(1);
     // rows modulo the range (see pass 1): a row has a place only where its class bit is set
     const u32 rlo32 = (u32)(g.lo + (w0 << g.wl)), mask = (nwr << g.wl) - 1;
-    u32* stage32 = reinterpret_cast<u32*>(stage);
-    __syncthreads();
-    const u32 rounds = s_rounds;
-    for (u32 g0 = 0; g0 < (u32)m; g0 += gs) {
-        const u32 g1 = min((u32)m, g0 + gs);
-        for (u32 i = tid; i < ((g1 - g0) * Lw + 1) / 2; i += kWinThreads)
+
+    for (u32 t = 0; t < T; ++t) {
+        const u32 m = (u32)min(kWinTile, g.n - t * kWinTile);
+        const u32 q1 = XS ? words_of(1 + t) : 0, Lw = q0 + q1;
+        auto load_next = [&]() {
+            if (t + 1 < T) {
+                load_class(2 + t);
+                load_cursors(t + 1);
+            }
+        };
+        if (Lw == 0) {  // nothing of this tile in the range
+            load_next();
+            continue;
+        }
+        // samples gathered at a time: all, or as many as fit (Lw <= 2 * 2048 words: at least one)
+        const u32 gs = m * Lw <= kStageWords ? m : kStageWords / Lw;
+        // (the stores of the tile before read only the gathered words)
+        b = max(a, b);
+        const Listing x0 = list_count(L, v, a, b, 0);
+        place_class(e1, 1 + t, q1 > 0, q0 * 64);
+        const bool edge = __syncthreads_or(at_edge(v, a, b));
+        for (u32 i = tid; i < (min(m, gs) * Lw + 1) / 2; i += kWinThreads)
             reinterpret_cast<uint4*>(stage)[i] = make_uint4(0u, 0u, 0u, 0u);
-        for (u32 rd = 0; rd < rounds; ++rd) {
-            const bool mine = (u32)tid >= g0 && (u32)tid < g1;
-            const u32 F = list_build(L, v, a, mine ? b : a, rd);
-            const u32 cw = (F + kWinThreads - 1) / kWinThreads * 32;  // a warp's share: whole steps of a piece a lane
-            const u32 f1 = min(F, (warp + 1) * cw);
-            u32 f = warp * cw + lane;
-            if (f < f1) {
-                Walk wk;
-                wk.init(L, v, f);
-                wk.to(L, v, f);
-                u32 nx[kRun];  // the next piece's values, loaded ahead
-                load_piece(v, wk, nx);
-                while (f < f1) {
-                    u32 x[kRun];
-                    #pragma unroll
-                    for (u32 i = 0; i < kRun; ++i) x[i] = nx[i];
-                    rows_of(x, wk.lo, wk.hi, rlo32, mask);
-                    const u32 at = (wk.k - g0) * 2 * Lw;
-                    f += 32;
-                    if (f < f1) {
-                        wk.to(L, v, f);
-                        load_piece(v, wk, nx);
-                    }
-                    #pragma unroll
-                    for (u32 i = 0; i < kRun; ++i) {
-                        // class 0 if two or more tiles hold the row, else the tile's
-                        // class if the row is kept there
-                        const u32 d = x[i], bit = 1u << (d & 31);
-                        uint2 e = e0[d >> 5];
-                        u32 to = at;
-                        if (!(e.x & bit)) {
-                            e = e1[d >> 5];
-                            to += 2 * q0;
-                        }
-                        if (e.x & bit) {
-                            const u32 rk = e.y + (u32)__popc(e.x & (bit - 1));
-                            atomicOr(stage32 + to + (rk >> 5), 1u << (rk & 31));
-                        }
+        const u32 F0 = list_place(L, v, x0);
+        const bool whole = !__syncthreads_or(gs < m || b - a > kRoundLen);
+        // the listed values into the gathered words of samples g0 on
+        auto gather = [&](u32 F, u32 g0) {
+            const u32 cs = (F + kWinThreads - 1) / kWinThreads * 32;  // a warp's share: whole steps of a piece a lane
+            const u32 f1 = min(F, (warp + 1) * cs);
+            u32 f = warp * cs + lane;
+            if (f >= f1) return;
+            Walk wk;
+            wk.init(L, f);
+            wk.to(L, f);
+            u32 nx[kRun];  // the next piece's values, loaded ahead
+            load_piece(v, wk, edge, nx);
+            while (f < f1) {
+                u32 x[kRun];
+                #pragma unroll
+                for (u32 i = 0; i < kRun; ++i) x[i] = nx[i];
+                rows_of(x, wk.lo, wk.hi, rlo32, mask);
+                u32* to = stage32 + (wk.k - g0) * 2 * Lw;
+                f += 32;
+                if (f < f1) {
+                    wk.to(L, f);
+                    load_piece(v, wk, edge, nx);
+                }
+                #pragma unroll
+                for (u32 i = 0; i < kRun; ++i) {
+                    // class 0 if two or more tiles hold the row, else the tile's
+                    // class if the row is kept there
+                    const u32 d = x[i], bit = 1u << (d & 31);
+                    uint2 e = e0[d >> 5];
+                    if (!(e.x & bit)) e = e1[d >> 5];
+                    if (e.x & bit) {
+                        const u32 rk = e.y + (u32)__popc(e.x & (bit - 1));
+                        atomicOr(to + (rk >> 5), 1u << (rk & 31));
                     }
                 }
             }
-            __syncthreads();  // the words are stored, or the list is rebuilt
+        };
+        // i / Lw by a multiplication (exact: i Lw < 2^32; Lw = 1 has no 32-bit reciprocal)
+        const u32 inv = Lw > 1 ? 0xffffffffu / Lw + 1 : 0;
+        for (u32 g0 = 0; g0 < m; g0 += gs) {
+            const u32 g1 = min(m, g0 + gs);
+            if (!whole && g0) {
+                __syncthreads();  // the words of the samples before are stored
+                for (u32 i = tid; i < (g1 - g0) * Lw; i += kWinThreads) stage[i] = 0ull;
+            }
+            int more = 1;
+            for (u32 rd = 0; more; ++rd) {
+                u32 F = F0;
+                if (whole) {
+                    more = 0;
+                } else {
+                    __syncthreads();  // the list before has been walked
+                    load_cursors(t);
+                    b = (u32)tid >= g0 && (u32)tid < g1 ? max(a, b) : a;
+                    const Listing x = list_count(L, v, a, b, rd);
+                    more = __syncthreads_or(b - a > (u64)(rd + 1) * kRoundLen);
+                    F = list_place(L, v, x);
+                    __syncthreads();
+                }
+                gather(F, g0);
+            }
+            __syncthreads();
+            if (g1 == m) load_next();
+            u64* dm = XM + (t * kWinTile + g0) * stride_m + s_at[0];
+            u64* ds = XS + (t * kWinTile + g0) * stride_s + s_at[1 + t];
+            for (u32 i = tid; i < (g1 - g0) * Lw; i += kWinThreads) {
+                const u32 y = Lw > 1 ? __umulhi(i, inv) : i, x = i - y * Lw;
+                u64* row = x < q0 ? dm + y * stride_m + x : ds + y * stride_s + (x - q0);
+                *row = stage[i];
+            }
         }
-        if (rounds == 0) __syncthreads();
-        u64* dm = XM + (k0 + g0) * stride_m + kbase[0] + s_rb[0];
-        u64* ds = XS + (k0 + g0) * stride_s + kbase[cl1] + s_rb[1];
-        for (u32 i = tid; i < (g1 - g0) * Lw; i += kWinThreads) {
-            const u32 y = Lw > 1 ? __umulhi(i, inv) : i, x = i - y * Lw;
-            u64* row = x < q0 ? dm + y * stride_m + x : ds + y * stride_s + (x - q0);
-            *row = stage[i];
-        }
-        __syncthreads();  // the gathered words are cleared for the next samples
     }
 }
 
@@ -646,7 +703,7 @@ cudaError_t launch_win_pack(const u64* ids, u64 N, const WinGeom& g, const u64* 
     const size_t smem = win_pack_smem(g);
     cudaError_t e = cudaFuncSetAttribute(k_win_pack, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_win_pack<<<(unsigned)(g.G * g.T), kWinThreads, smem, st>>>(values_of(ids, N), g, cls, pre, cnt, boff, curs, kbase, XM,
+    k_win_pack<<<(unsigned)g.G, kWinThreads, smem, st>>>(values_of(ids, N), g, cls, pre, cnt, boff, curs, kbase, XM,
                                                                  stride_m, XS, stride_s);
     return cudaGetLastError();
 }
