@@ -294,16 +294,32 @@ int all_pairs_impl(jsim_ctx* ctx, const jsim_sets* sets, void* C, uint64_t* size
     // values lie in [minid, maxid]; batches are aligned to multiples of m~ and
     // empty stretches of the value range are skipped
     u64 mt = 0, b_beg = 0, b_end = 0;
-    partition_rows(st.N ? st.minid : 0, st.N ? st.maxid : 0, ctx->opt.batch_rows, part, parts, b_beg, b_end, mt);
-    ctx->stats.batch_rows = mt;
+    const u64 v0 = st.N ? st.minid : 0, v1 = st.N ? st.maxid : 0;
+    // (a part keeps the width jsim_partition_batches cuts the batches by)
+    u64 width = parts == 1 && !counts_only ? dense_batch_rows(ctx, n, st.N, v0, v1) : ctx->opt.batch_rows;
+    partition_rows(v0, v1, width, part, parts, b_beg, b_end, mt);
     int variant = ctx->opt.variant;
     if (st.N && b_beg < b_end) {
         BatchBufs bb;
         u64 lo = b_beg * mt;
+        const jsim_stats before = ctx->stats;
         for (;;) {
+            ctx->stats.batch_rows = mt;
             u64 R = 0, stride = 0, next = 0;
             bool has_next = false;
             rc = build_batch(ctx, st, bb, lo, mt, R, stride, nullptr, &has_next, &next);
+            if (rc == JSIM_ERR_OOM && width != ctx->opt.batch_rows && mt > auto_batch_rows(~0ull)) {
+                // no room for the wide batches: from the start again in the
+                // widest ones that stay in L2
+                width = auto_batch_rows(~0ull);
+                partition_rows(v0, v1, width, part, parts, b_beg, b_end, mt);
+                lo = b_beg * mt;
+                for (DevBuf* b : {&bb.bitmap, &bb.seen, &bb.dir, &bb.X}) b->release();
+                CK(cudaMemsetAsync(Cacc.p, 0, n * n * cb, ctx->stream));
+                if (ctx->opt.count_useful) CK(cudaMemsetAsync(useful.p, 0, sizeof(u64), ctx->stream));
+                ctx->stats = before;
+                continue;
+            }
             if (rc) return rc;
             if (R) {
                 const u64 W = (R + 63) / 64;
@@ -322,6 +338,8 @@ int all_pairs_impl(jsim_ctx* ctx, const jsim_sets* sets, void* C, uint64_t* size
             if (!has_next || next / mt >= b_end) break;
             lo = next / mt * mt;
         }
+    } else {
+        ctx->stats.batch_rows = mt;
     }
 
     // nothing is written when a bounded device wait ran out

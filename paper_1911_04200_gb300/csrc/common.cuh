@@ -49,7 +49,7 @@ struct Plan {
                  // validation) and the windowed ingest's count of class rows, zeroed by the plan
 };
 constexpr u64 kPlanTotals = 8;
-constexpr int kTicketFilter = 4, kTicketPack = 5, kTicketValidate = 6;
+constexpr int kTicketFilter = 4, kTicketPack = 5, kTicketValidate = 6, kTicketRank = 6;  // (validation has a plan of its own)
 constexpr int kPlanRowsTotal = 7;
 // u64 words of a plan over n samples: beg, len, cofs (n + 1), totals
 __host__ __device__ inline u64 plan_words(u64 n) { return 3 * n + 1 + kPlanTotals; }
@@ -117,12 +117,19 @@ cudaError_t launch_validate(const u64* offsets, const u64* ids, u64 n, Plan plan
 // width/32 u32 words each, tile-major); twice likewise (optional).
 cudaError_t launch_filter_tiles(const u64* ids, u64 n, Plan plan, u64 max_chunks, u64 lo, u64 width,
                                u32* bitmaps, u32* twice, const u32* tile_of, int sms, cudaStream_t st);
+// Every value's row number among the kept rows of a batch (bitmap, dir, boff)
+// into ranks[its position] (~0: not kept), and every tile's bitmap over those
+// rows (zeroed before; tile_words u32 words apart).
+cudaError_t launch_rank_tiles(const u64* ids, u64 n, Plan plan, u64 max_chunks, u64 lo, u64 width, const u64* bitmap,
+                              const u32* dir, const u64* boff, u32* ranks, u32* tiles, const u32* tile_of,
+                              u64 tile_words, int sms, cudaStream_t st);
 // Single pass into both matrices: class-0 values to XM (null: there are
-// none), class cls_of[i] values to XS, atomically OR-ed.
-cudaError_t launch_pack_classes(const u64* ids, u64 n, Plan plan, u64 max_chunks, u64 lo, u64 width, const u64* cls,
-                                const u32* dir, const u64* boff, u64 nwords, const u64* kbase, const u32* cls_of,
-                                const u32* row_of, u64* XM, u64 stride_m, u64* XS, u64 stride_s, int sms,
-                                cudaStream_t st);
+// none), class cls_of[i] values to XS, atomically OR-ed.  With ranks, the
+// class bitmaps are over the rows launch_rank_tiles numbered.
+cudaError_t launch_pack_classes(const u64* ids, const u32* ranks, u64 n, Plan plan, u64 max_chunks, u64 lo, u64 width,
+                                const u64* cls, const u32* dir, const u64* boff, u64 nwords, const u64* kbase,
+                                const u32* cls_of, const u32* row_of, u64* XM, u64 stride_m, u64* XS, u64 stride_s,
+                                int sms, cudaStream_t st);
 // twice (optional): also the bitmap of rows held by two or more samples
 cudaError_t launch_filter(const u64* ids, u64 n, Plan plan, u64 max_chunks, u64 lo, u64 width,
                           u32* bitmap, int sms, cudaStream_t st, u32* twice = nullptr);

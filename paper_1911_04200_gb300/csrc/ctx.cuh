@@ -476,6 +476,49 @@ u64 auto_batch_rows(u64 domain)
     return m;
 }
 
+// Rows per batch of a whole dense call, and the time its ingest takes (*ms).
+// A batch costs kDenseBatchMs whatever it holds (launches, the directory, the
+// host's look at its row count); a value costs more in a wider batch, whose
+// bitmap and directory no longer stay in L2 (kDenseValueMs: 2^28 rows and
+// fewer, 2^29, ... 2^32).  Measured on clade samples over [0, 2^32), call less
+// product in ms at 2^28 / 2^29 / 2^30 / 2^31 / 2^32 rows, and the model:
+//   1.4e7 values   2.9 / 1.9 / 1.6 / 1.3 / 1.4    3.1 / 1.8 / 1.4 / 1.3 / 1.3
+//   4.2e7          3.9 / 2.8 / 2.7 / 3.1 / 3.6    3.9 / 2.8 / 2.8 / 3.3 / 3.6
+//   1.4e8          6.5 / 6.2 / 7.9 / 10  / 12     6.6 / 6.1 / 7.7 / 10  / 12
+//   4.2e8         13.7 / 15.9 / 23 / 29          14.5 / 15.6 / 22 / 30
+// So few values take wide batches and many take 2^28 rows.  A batch is wider
+// than 2^28 only where its packed matrix is small (bounded by its values) and
+// the device has room for its bitmaps.
+constexpr double kDenseBatchMs = 0.17;
+constexpr double kDenseValueMs[2][5] = {{2.8e-8, 3.4e-8, 5.0e-8, 7.0e-8, 8.2e-8},   // one filter
+                                        {2.8e-8, 3.9e-8, 6.1e-8, 8.2e-8, 9.8e-8}};  // two-or-more
+u64 dense_batch_rows(const jsim_ctx* ctx, u64 n, u64 N, u64 minid, u64 maxid, double* ms = nullptr)
+{
+    const u64 span = maxid - minid;
+    const double* value_ms = kDenseValueMs[ctx->opt.filter_min == 2];
+    auto cost = [&](u64 w, int k) {
+        return (double)(maxid / w - minid / w + 1) * kDenseBatchMs + (double)N * value_ms[k];
+    };
+    u64 best = ctx->opt.batch_rows ? ctx->opt.batch_rows : auto_batch_rows(span + 1 ? span + 1 : ~0ull);
+    double best_ms = cost(best, 0);
+    size_t free_b = 0, total_b = 0;
+    for (int k = 1; k < 5 && !ctx->opt.batch_rows; ++k) {
+        const u64 w = 1ull << (28 + k);
+        if (w / 2 > span) break;
+        const double t = cost(w, k);
+        if (t >= best_ms) continue;
+        const double held = std::min(1.0, (double)w / ((double)span + 1.0)) * (double)N;
+        const double x_bytes = (double)round_up(std::max<u64>(n, 1), kRowPad) * held / 8.0;
+        const double bytes = x_bytes + (double)w / 8.0 * (ctx->opt.filter_min == 2 ? 2.5 : 1.5);
+        if (!total_b && cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) { cudaGetLastError(); break; }
+        if (x_bytes > (double)(4ull << 30) || bytes > (double)free_b / 4.0) continue;
+        best = w;
+        best_ms = t;
+    }
+    if (ms) *ms = best_ms;
+    return best;
+}
+
 // Variant choice, from a sweep on GB300 (random packed words, Tbit-ops/s):
 //   n      64    128   192   256   512   1024  2048
 //   POPC   71    92    104   111   123   130   142

@@ -35,8 +35,9 @@
 // Every count is the same integer as the dense product's (a sum over the
 // same rows, Eq. 4, grouped differently), so C and J are bit-identical.  With
 // AUTO the sketch's own rows are classified first, and the call goes on dense
-// unless the estimated time of the whole call (product and ingest at rates
-// measured on GB300) is at least 5 % below the dense call's.
+// unless the order leaves well below the dense product and the estimated time
+// of the whole call (product and ingest at rates measured on GB300) is no more
+// than the dense call's.
 //
 // Internal header of the C-ABI translation unit (included once, after ctx.cuh).
 #pragma once
@@ -49,24 +50,54 @@ constexpr u64 kMaxTiles = 16;             // n <= 2048
 constexpr u64 kSketchPerSample = 512;     // values per sample in the sketch range, on average
 constexpr u64 kMinClassRows = 1ull << 18; // batch width granule: one scan block of every class
 constexpr u64 kTileBitmapBytes = 128ull << 20;  // all tiles' filter bitmaps of a batch together
-// Rates measured on GB300 (1024 clade samples, 1.3e9 values; both filters)
-// that the automatic choice weighs: dense SM-pair product and block-sparse
-// products in bit-operations per ms; ingest (validation, filter, scan, pack)
-// per value in ms, dense and block-sparse, one filter and two-or-more.
-// Batch widths swept at 2^25..2^28 rows (with the samples planned in tile
-// order, so only one or two tiles' structures are in use at a time): 62.8 /
-// 58.4 / 61.4 ms per call at 2^26 / 2^27 / 2^28 rows with one filter, 69.6 /
-// 61.9 / 62.3 ms at 2^25 / 2^26 / 2^27 with the two-or-more filter - the
-// widths where all tiles' bitmaps take kTileBitmapBytes.
-constexpr double kDenseBitopsPerMs = 1.1e12;
-constexpr double kSparseBitopsPerMs = 0.75e12;
-constexpr double kIngestDenseMs[2] = {2.8e-8, 2.5e-8};
-constexpr double kIngestSparseMs[2] = {2.8e-8, 3.4e-8};
+// Per-value ingest, batch widths swept at 2^25..2^28 rows (with the samples
+// planned in tile order, so only one or two tiles' structures are in use at a
+// time; 1024 clade samples, 1.3e9 values): 62.8 / 58.4 / 61.4 ms per call at
+// 2^26 / 2^27 / 2^28 rows with one filter, 69.6 / 61.9 / 62.3 ms at 2^25 /
+// 2^26 / 2^27 with the two-or-more filter - the widths where all tiles'
+// bitmaps take kTileBitmapBytes.
+//
+// Times the automatic choice weighs, measured on GB300 over clade samples in
+// [0, 2^32) (n = 300 .. 2048, 7.9e6 .. 1.3e9 values).  Products, in
+// multiply-adds of whole tiles per ms: the SM-pair product's 256 x 256 tiles,
+// the diagonal 128 x 128 tiles.  Ingest: the ranked ingest takes what the
+// dense call's takes (dense_batch_rows); the windowed ingest kWinTileMs for
+// every tile over 2^32 rows and kWinValueMs a value; the per-value ingest
+// kPerBatchMs a batch whatever it holds and kPerValueMs a value.  Page-locked
+// input fed in pieces arrives at kLinkMs a value, beside the sparse batches
+// and before the dense ones.  Whole calls in ms, n = 1024:
+//   values       1.4e7      4.2e7      1.4e8      4.2e8
+//   dense        2.1        4.8        13.0       33.6
+//   ranked       2.7        4.1         7.5
+//   windowed                10.2       11.4       14.6
+//   per value    9.6
+constexpr double kPairMacsPerMs = 3.8e12;
+constexpr double kDiagMacsPerMs = 2.3e12;
+constexpr double kPerBatchMs[2] = {0.24, 0.18};  // one filter, two-or-more
+constexpr double kPerValueMs = 2.0e-8;
+constexpr double kWinTileMs[2] = {1.2, 1.42};
+constexpr double kWinValueMs[2] = {0.75e-8, 1.3e-8};
+constexpr double kLinkMs = 4.7e-8;
+double pair_product_ms(u64 n, double rows)
+{
+    const double tt = (double)((n + 255) / 256);
+    return tt * (tt + 1.0) / 2.0 * 65536.0 * rows / kPairMacsPerMs;
+}
+// What the sketch and the order of the samples take before the first batch.
+double sketch_ms(u64 n) { return 0.3 + 0.75e-6 * (double)n * (double)n; }
+// Ranked ingest: at most this many values (a 32-bit row number is kept for
+// each: 4 GiB).
+constexpr u64 kRankMaxValues = 1ull << 30;
 // Windowed ingest (windows.cu): windows of 2^kWinLog rows, used where a
 // sample has kWinMinValues values in a window on average (below, most of a
 // range's work would go to samples with no value in it).
 constexpr int kWinLog = 16;
 constexpr double kWinMinValues = 0.5;
+// From this density the windowed ingest is taken whatever the other would
+// cost: over 2^32 rows the two cross at 4 to 5 values a window (1024 samples,
+// 2.1 a window: 11.4 ms windowed, 7.5 ranked; 6.2: 14.6 windowed, and the
+// ranked ingest alone would take 14).
+constexpr double kWinSureValues = 3.0;
 constexpr u64 kWinMaxBatch = 1ull << 30;
 
 // Row classes from the tiles' bitmaps: class 0 = rows of two or more tiles,
@@ -270,10 +301,58 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
     const int wl = kWinLog;
     const double per_window =
         st.N ? (double)st.N / (double)n / ((double)span + 1.0) * (double)(1ull << wl) : 0.0;
-    const bool windowed = per_window >= kWinMinValues && !feed;
-    const u64 mt = feed ? feed->mt : sparse_batch_rows(ctx, n, span, windowed);
+    // Ranked ingest: the call's row bitmap over the whole value range, as the
+    // dense path builds it, numbers the nonzero rows, and the tiles' bitmaps
+    // and the classes are over those row numbers only.  A thin value range
+    // then pays for its rows, not for every tile's copy of the range; taken
+    // where the model says so, and in place of the per-value ingest wherever
+    // the batches' width is free.
+    double dense_ingest = 0;
+    const u64 dense_mt = st.N ? dense_batch_rows(ctx, n, st.N, st.minid, st.maxid, &dense_ingest) : 0;
+    const double windowed_ms = ((double)span + 1.0) / 4294967296.0 * (double)T * kWinTileMs[twice] +
+                               (double)st.N * kWinValueMs[twice];
+    bool windowed = false, ranked = !feed && st.N && st.N <= kRankMaxValues && !ctx->opt.batch_rows;
+    u64 mt = 0;
+    double sparse_ingest = 0;
+    auto choose_ingest = [&]() {
+        windowed = per_window >= kWinMinValues && !feed;
+        if (ranked && windowed && (per_window >= kWinSureValues || windowed_ms <= dense_ingest)) ranked = false;
+        if (ranked) windowed = false;
+        mt = feed ? feed->mt : ranked ? std::max(kMinClassRows, dense_mt) : sparse_batch_rows(ctx, n, span, windowed);
+        sparse_ingest = ranked     ? dense_ingest
+                        : windowed ? windowed_ms
+                        : mt       ? (double)(st.maxid / mt - st.minid / mt + 1) * kPerBatchMs[twice] +
+                                   (double)st.N * kPerValueMs
+                                   : 0.0;
+    };
+    choose_ingest();
     if (!mt) return JSIM_ERR_UNSUPPORTED;
     ctx->stats.batch_rows = mt;
+    // The call's time dense with `rows` nonzero rows, and block-sparse with
+    // `prod` ms of products.  A value is at most one row (with the two-or-more
+    // filter two values are), and where even that many rows multiply faster
+    // dense than the sparse ingest takes, there is nothing a sketch could tell.
+    const double link = feed ? (double)st.N * kLinkMs : 0.0;
+    auto dense_ms = [&](double rows) { return link + dense_ingest + pair_product_ms(n, rows); };
+    auto sparse_ms = [&](double prod) { return std::max(link, sparse_ingest) + prod; };
+    if (may_decline && st.N && !feed &&
+        dense_ms((double)st.N / (twice ? 2.0 : 1.0)) <= sketch_ms(n) + sparse_ms(0.0)) {
+        declined = true;
+        return JSIM_OK;
+    }
+    DevBuf rk_bits, rk_seen, rk_dir, rk_bsum, rk_boff, ranks;
+    if (ranked) {
+        const u64 nw = mt / 64, nb = (nw + kScanBlockWords - 1) / kScanBlockWords;
+        ranked = rk_bits.ensure(ctx, nw * 8) && (!twice || rk_seen.ensure(ctx, nw * 8)) && rk_dir.ensure(ctx, nw * 4) &&
+                 rk_bsum.ensure(ctx, nb * 8) && rk_boff.ensure(ctx, nb * 8) && ranks.ensure(ctx, st.N * 4);
+        if (!ranked) {  // no room for it: the other ingests hold less
+            for (DevBuf* b : {&rk_bits, &rk_seen, &rk_dir, &rk_bsum, &rk_boff, &ranks}) b->release();
+            choose_ingest();
+            if (!mt) return JSIM_ERR_UNSUPPORTED;
+            ctx->stats.batch_rows = mt;
+        }
+    }
+
     // search bounds of a batch at lo: with a feed, the slices of lo's piece
     const u64* pb = st.d_off;
     const u64* pe = nullptr;
@@ -304,6 +383,7 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
         DevBuf B, B2, cls, dir, bsum, boff, Rd, plan_buf, cnt, curs, gcurs, pre;
         Plan plan{};
         WinGeom g{};
+        u64 nw = 0;                    // words of a class bitmap
         cudaEvent_t done = nullptr;    // totals on the host
         cudaEvent_t packed = nullptr;  // the last pack that read the slot's structures
         bool pack_pending = false;
@@ -316,7 +396,7 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
     const u64 nwin_max = mt >> wl;
     const u64 ranges_max = nwin_max;  // a range holds one window or more
     for (Slot& x : slot) {
-        ALLOC(x.cls, (T + 1) * nw_max * sizeof(u64));
+        if (!ranked) ALLOC(x.cls, (T + 1) * nw_max * sizeof(u64));
         if (windowed) {
             ALLOC(x.B, T * nw_max * sizeof(u64));
             if (twice) ALLOC(x.B2, T * nw_max * sizeof(u64));
@@ -327,7 +407,7 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
             const WinGeom wg = win_geom(n, T, 0, mt, wl, twice);
             ALLOC(x.curs, (wg.G + 1) * n * sizeof(u64));
             ALLOC(x.gcurs, (wg.NG + 1) * n * sizeof(u64));
-        } else {
+        } else if (!ranked) {
             ALLOC(x.B, T * nw_max * sizeof(u64));
             if (twice) ALLOC(x.B2, T * nw_max * sizeof(u64));
             ALLOC(x.dir, (T + 1) * nw_max * sizeof(u32));
@@ -420,30 +500,59 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
             CK(cudaEventRecord(x.done, ccs));
             return JSIM_OK;
         }
+        u64 cw = nw;  // words of a class bitmap
+        const u64* B2 = twice ? x.B2.as<u64>() : nullptr;
         {
             StageTimer t(ctx, &ctx->stats.ms_filter);
             // the plan lists the samples in their order (entry k: the sample
             // at position k), so the chunks in flight belong to one or two
             // tiles and their bitmaps and directories stay in L2
             CK(launch_plan(pb, st.d_ids, n, lo, hi, false, x.plan, cs, d_order.as<u32>(), pe));
-            CK(cudaMemsetAsync(x.B.p, 0, T * nw * sizeof(u64), cs));
-            if (twice) CK(cudaMemsetAsync(x.B2.p, 0, T * nw * sizeof(u64), cs));
-            CK(launch_filter_tiles(st.d_ids, n, x.plan, st.max_chunks, lo, width, x.B.as<u32>(),
-                                   twice ? x.B2.as<u32>() : nullptr, d_tile.as<u32>(), ctx->sms, cs));
+            if (ranked) {
+                CK(cudaMemsetAsync(rk_bits.p, 0, nw * sizeof(u64), cs));
+                if (twice) CK(cudaMemsetAsync(rk_seen.p, 0, nw * sizeof(u64), cs));
+                CK(launch_filter(st.d_ids, n, x.plan, st.max_chunks, lo, width,
+                                 twice ? rk_seen.as<u32>() : rk_bits.as<u32>(), ctx->sms, cs,
+                                 twice ? rk_bits.as<u32>() : nullptr));
+                CK(launch_scan(rk_bits.as<u64>(), nw, rk_dir.as<u32>(), rk_bsum.as<u64>(), rk_boff.as<u64>(),
+                               x.Rd.as<u64>(), cs));
+                CK(cudaMemcpyAsync(hs + 17, x.Rd.p, sizeof(u64), cudaMemcpyDeviceToHost, cs));
+                CK(cudaStreamSynchronize(cs));
+                // kept rows hold two samples or more already (twice): which
+                // tiles hold them is all the classes need
+                cw = std::max<u64>(1, (hs[17] / 64 + kScanBlockWords) / kScanBlockWords) * kScanBlockWords;
+                B2 = nullptr;
+                ALLOC(x.B, T * cw * sizeof(u64));
+                ALLOC(x.cls, (T + 1) * cw * sizeof(u64));
+                ALLOC(x.dir, (T + 1) * cw * sizeof(u32));
+                ALLOC(x.bsum, (T + 1) * cw / kScanBlockWords * sizeof(u64));
+                ALLOC(x.boff, ((T + 1) * cw / kScanBlockWords + 1) * sizeof(u64));
+                CK(cudaMemsetAsync(x.B.p, 0, T * cw * sizeof(u64), cs));
+                CK(launch_rank_tiles(st.d_ids, n, x.plan, st.max_chunks, lo, width, rk_bits.as<u64>(),
+                                     rk_dir.as<u32>(), rk_boff.as<u64>(), ranks.as<u32>(), x.B.as<u32>(),
+                                     d_tile.as<u32>(), 2 * cw, ctx->sms, cs));
+                ctx->stats.launches += 3;
+            } else {
+                CK(cudaMemsetAsync(x.B.p, 0, T * nw * sizeof(u64), cs));
+                if (twice) CK(cudaMemsetAsync(x.B2.p, 0, T * nw * sizeof(u64), cs));
+                CK(launch_filter_tiles(st.d_ids, n, x.plan, st.max_chunks, lo, width, x.B.as<u32>(),
+                                       twice ? x.B2.as<u32>() : nullptr, d_tile.as<u32>(), ctx->sms, cs));
+            }
             // one word per thread: short CTAs that any free slot can take
-            k_classify<<<(unsigned)std::max<u64>(1, (nw + 255) / 256), 256, 0, cs>>>(
-                x.B.as<u64>(), twice ? x.B2.as<u64>() : nullptr, T, nw, x.cls.as<u64>());
+            k_classify<<<(unsigned)std::max<u64>(1, (cw + 255) / 256), 256, 0, cs>>>(x.B.as<u64>(), B2, T, cw,
+                                                                                    x.cls.as<u64>());
             CK(cudaGetLastError());
             ctx->stats.launches += 3;
         }
+        x.nw = cw;
         {
             StageTimer t(ctx, &ctx->stats.ms_scan);
-            CK(launch_scan(x.cls.as<u64>(), (T + 1) * nw, x.dir.as<u32>(), x.bsum.as<u64>(), x.boff.as<u64>(),
+            CK(launch_scan(x.cls.as<u64>(), (T + 1) * cw, x.dir.as<u32>(), x.bsum.as<u64>(), x.boff.as<u64>(),
                            x.Rd.as<u64>(), cs));
             ctx->stats.launches += 2;
         }
         // every class's first block offset, the total and the plan's next value
-        const u64 nb = nw / kScanBlockWords;
+        const u64 nb = cw / kScanBlockWords;
         CK(cudaMemcpy2DAsync(hs, sizeof(u64), x.boff.as<u64>(), nb * sizeof(u64), sizeof(u64), T + 1,
                              cudaMemcpyDeviceToHost, cs));
         CK(cudaMemcpyAsync(hs + 17, x.Rd.p, sizeof(u64), cudaMemcpyDeviceToHost, cs));
@@ -544,26 +653,22 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
             if (rc) return rc;
             rc = read_classify(0, hn, nx);
             if (rc) return rc;
-            // the call's product work, dense and block-sparse, scaled from the
-            // sketch range's rows by values; with the ingest, the call's time
-            // either way at the measured rates
-            double rows = 0, sparse = 0;
+            // the call's time either way, its rows scaled from the sketch
+            // range's by values
+            double kept = 0, own = 0;
             for (u64 c = 0; c <= T; ++c) {
-                const double r = (double)Rc[c];
-                rows += r;
-                if (c == 0) {
-                    sparse += r * (double)n * (double)(n + 1) / 2.0;
-                } else {
-                    const double m = (double)std::min<u64>(kTile, n - (c - 1) * kTile);
-                    sparse += r * m * (m + 1) / 2.0;
-                }
+                kept += (double)Rc[c];
+                if (c) own += (double)Rc[c];
             }
             const double scale = range_values ? (double)st.N / (double)range_values : 1.0;
-            const double dense_bitops = rows * scale * (double)n * (double)(n + 1) / 2.0;
-            const double sparse_bitops = sparse * scale;
-            const double t_dense = dense_bitops / kDenseBitopsPerMs + (double)st.N * kIngestDenseMs[twice];
-            const double t_sparse = sparse_bitops / kSparseBitopsPerMs + (double)st.N * kIngestSparseMs[twice];
-            if (t_sparse > 0.95 * t_dense) {
+            // (Rc is what the sparse products multiply, windowed ingest rounds
+            // it up per range; the dense product multiplies the rows themselves)
+            const double rows = (double)range_rows * scale;
+            const double prod_sparse = pair_product_ms(n, (kept - own) * scale) +
+                                       own * scale * (double)(kTile * kTile) / kDiagMacsPerMs;
+            // an order that empties few blocks is no reason to go on: what is
+            // left of the gain does not carry the classes
+            if (prod_sparse > 0.6 * pair_product_ms(n, rows) || sparse_ms(prod_sparse) > dense_ms(rows)) {
                 declined = true;
                 ctx->stats.windows = 0;
                 return JSIM_OK;
@@ -662,7 +767,6 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
             if (rc) return rc;
             dense_run = has_next && next / mt * mt == lo_sp;
             const Slot& x = slot[si];
-            const u64 nw = mt / 64;
             std::vector<u64> W(T + 1);
             u64 R = 0, Wmax_s = 0;
             bool full = false;
@@ -730,10 +834,11 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
                                                           Wc.as<u64>(), 1);
                         CK(cudaGetLastError());
                     }
-                    CK(launch_pack_classes(st.d_ids, n, x.plan, st.max_chunks, lo, mt, x.cls.as<u64>(),
-                                           x.dir.as<u32>(), x.boff.as<u64>(), nw, kbase.as<u64>(),
-                                           d_cls_of.as<u32>(), d_rowk.as<u32>(), W[0] ? XM.as<u64>() : nullptr,
-                                           stride_m, Wmax_s ? XS.as<u64>() : nullptr, stride_s, ctx->sms, cs));
+                    CK(launch_pack_classes(st.d_ids, ranked ? ranks.as<u32>() : nullptr, n, x.plan, st.max_chunks, lo,
+                                           ranked ? 64 * x.nw : mt, x.cls.as<u64>(), x.dir.as<u32>(),
+                                           x.boff.as<u64>(), x.nw, kbase.as<u64>(), d_cls_of.as<u32>(),
+                                           d_rowk.as<u32>(), W[0] ? XM.as<u64>() : nullptr, stride_m,
+                                           Wmax_s ? XS.as<u64>() : nullptr, stride_s, ctx->sms, cs));
                     ctx->stats.launches += 3;
                 }
                 totM += W[0];
