@@ -31,9 +31,6 @@ struct jsim_ctx {
     char cuda_err[256];
     // small pinned host scratch (256 u64) for device <-> host scalars
     unsigned long long* h_scalars;
-    // page-locked scratch for the block-sparse path's sketch similarities (grown on demand)
-    void* h_sketch = nullptr;
-    size_t h_sketch_bytes = 0;
     // the block-sparse path's classification stream, at the device's highest priority (created on demand)
     cudaStream_t class_stream = nullptr;
     // device error word of kernels with bounded waits

@@ -83,8 +83,9 @@ double pair_product_ms(u64 n, double rows)
     const double tt = (double)((n + 255) / 256);
     return tt * (tt + 1.0) / 2.0 * 65536.0 * rows / kPairMacsPerMs;
 }
-// What the sketch and the order of the samples take before the first batch.
-double sketch_ms(u64 n) { return 0.3 + 0.75e-6 * (double)n * (double)n; }
+// What the order of the samples takes, and with the sketch before it.
+double order_ms(u64 n) { return 0.05 + 0.7e-3 * (double)n; }
+double sketch_ms(u64 n) { return 0.2 + order_ms(n); }
 // Ranked ingest: at most this many values (a 32-bit row number is kept for
 // each: 4 GiB).
 constexpr u64 kRankMaxValues = 1ull << 30;
@@ -174,7 +175,7 @@ unsigned grid_of(u64 items, int sms, unsigned threads)
 // Sketch counts are far below 2^24, so c and u are exact floats and c / u is
 // one correctly rounded division.
 template <typename CT>
-__global__ void k_sketch_j(const CT* __restrict__ Cs, u64 n, float* __restrict__ Jf, u64* __restrict__ sz)
+__global__ void k_sketch_j(const CT* __restrict__ Cs, u64 n, float* __restrict__ Jf, u64 stride, u64* __restrict__ sz)
 {
     for (u64 t = blockIdx.x * (u64)blockDim.x + threadIdx.x; t < n * n; t += (u64)gridDim.x * blockDim.x) {
         const u64 i = t / n, j = t - i * n;
@@ -184,7 +185,7 @@ __global__ void k_sketch_j(const CT* __restrict__ Cs, u64 n, float* __restrict__
             const float c = (float)Cs[a * n + b], u = (float)Cs[i * n + i] + (float)Cs[j * n + j] - c;
             v = u > 0.f ? __fdiv_rn(c, u) : 0.f;
         }
-        Jf[t] = v;
+        Jf[i * stride + j] = v;
         if (i == j) sz[i] = (u64)Cs[t];
     }
 }
@@ -194,42 +195,98 @@ __global__ void k_sketch_j(const CT* __restrict__ Cs, u64 n, float* __restrict__
 // the unplaced one with the largest J to any sample already in the current
 // tile of kTile (a new tile starts from its predecessor's similarities);
 // ties go to the smaller index, and a sample sharing nothing with the tile
-// is taken largest first.  Each step is one pass: the scores take in the
-// last placed sample's similarities and the best unplaced sample is found
-// in the same loop.
-std::vector<u32> sample_order(const float* Jm, const u64* sz, u64 n)
+// is taken largest first.  Writes the order, its inverse and, per position,
+// the tile, class and row of its sample; null Jm: the samples as they come.
+//
+// One CTA, bound by the n - 1 dependent steps: a row of Jm from L2 (the last
+// placed sample's), the running scores in registers, and one maximum over the
+// CTA with a single barrier (warp maxima by redux, shared slots of alternating
+// steps).  Eight warps with PER samples a thread, loaded four at a time: more
+// warps issue more of the same instructions per step.  The same chain on the
+// host, with Jm and sizes copied out and the order copied in, took 3.5 ms for
+// 2048 samples and 0.9 ms for 1024; here
+// 1.6 ms and 0.65 ms.
+constexpr int kOrderThreads = 256;
+template <int PER>
+__global__ void __launch_bounds__(kOrderThreads)
+k_sample_order(const float* __restrict__ Jm, u32 stride, const u64* __restrict__ sz, u32 n, u32* order, u32* pos,
+               u32* tile, u32* cls_of, u32* rowk)
 {
-    std::vector<u32> order;
-    order.reserve(n);
-    std::vector<char> placed(n, 0);
-    std::vector<float> score(n, 0.f);
-    u64 first = 0;
-    for (u64 i = 1; i < n; ++i)
-        if (sz[i] > sz[first]) first = i;
-    order.push_back((u32)first);
-    placed[first] = 1;
-    for (u64 step = 1; step < n; ++step) {
-        // the scores: J to the current tile's samples (a new tile: to its
-        // predecessor only), with the last placed sample taken in now
-        const float* r = Jm + (u64)order.back() * n;
-        const bool fresh = step == 1 || step % kTile == 0;
-        u64 best = n;
-        float bs = 0.f;
-        for (u64 j = 0; j < n; ++j) {
-            const float v = fresh ? r[j] : std::max(score[j], r[j]);
-            score[j] = v;
-            if (!placed[j] && v > bs) {
-                bs = v;
-                best = j;
+    static_assert(PER % 4 == 0, "16-byte loads");
+    constexpr int kWarps = kOrderThreads / 32;
+    __shared__ uint2 s_best[2][kWarps];
+    const u32 t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    for (u32 k = t; k < n; k += kOrderThreads) {
+        tile[k] = k / (u32)kTile;
+        cls_of[k] = 1 + k / (u32)kTile;
+        rowk[k] = k;
+        if (!Jm) order[k] = pos[k] = k;
+    }
+    if (!Jm) return;
+    // element e of a thread is sample 4 t + e % 4 + 1024 (e / 4)
+    auto sample = [&](int e) { return 4 * t + (u32)(e & 3) + (u32)(e >> 2) * 4 * kOrderThreads; };
+    u32 size[PER];  // + 1; 0: placed, or past the last sample
+    float score[PER];
+    #pragma unroll
+    for (int e = 0; e < PER; ++e) {
+        const u32 j = sample(e);
+        size[e] = j < n ? (u32)min(sz[j], (u64)0xfffffffe) + 1u : 0u;
+        score[e] = 0.f;
+    }
+    u32 par = 0;
+    // the largest v over the CTA (0: none) and the smallest sample that has it
+    auto best = [&](const u32 (&v)[PER], u32& bv) -> u32 {
+        u32 mv = v[0], mj = 0;
+        #pragma unroll
+        for (int e = 1; e < PER; ++e)
+            if (v[e] > mv) {
+                mv = v[e];
+                mj = (u32)e;
+            }
+        mj = 4 * t + (mj & 3) + (mj >> 2) * 4 * kOrderThreads;
+        const u32 wv = __reduce_max_sync(0xffffffffu, mv);
+        const u32 wj = __reduce_min_sync(0xffffffffu, mv == wv ? mj : ~0u);
+        if (lane == 0) s_best[par][warp] = make_uint2(wv, wj);
+        __syncthreads();
+        const uint2 c = s_best[par][lane & (kWarps - 1)];
+        par ^= 1u;
+        bv = __reduce_max_sync(0xffffffffu, c.x);
+        return __reduce_min_sync(0xffffffffu, c.x == bv ? c.y : ~0u);
+    };
+    u32 bv, last = best(size, bv);
+    for (u32 step = 0;; ++step) {
+        float4 row[PER / 4];
+        if (step + 1 < n) {
+            #pragma unroll
+            for (int q = 0; q < PER / 4; ++q) {
+                const u32 j = sample(4 * q);
+                row[q] = j < n ? *(const float4*)(Jm + (u64)last * stride + j) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
         }
-        if (best == n)
-            for (u64 j = 0; j < n; ++j)
-                if (!placed[j] && (best == n || sz[j] > sz[best])) best = j;
-        order.push_back((u32)best);
-        placed[best] = 1;
+        if (((last >> 2) & (kOrderThreads - 1)) == t) {
+            #pragma unroll
+            for (int e = 0; e < PER; ++e)
+                if (last == sample(e)) size[e] = 0;
+            order[step] = last;
+            pos[last] = step;
+        }
+        if (step + 1 >= n) break;
+        // the scores: J to the current tile's samples (a new tile: to its
+        // predecessor only), with the last placed sample taken in now
+        if (step == 0 || (step + 1) % (u32)kTile == 0) {
+            #pragma unroll
+            for (int e = 0; e < PER; ++e) score[e] = 0.f;
+        }
+        u32 v[PER];
+        #pragma unroll
+        for (int e = 0; e < PER; ++e) {
+            const float4 r = row[e >> 2];
+            score[e] = fmaxf(score[e], (e & 3) == 0 ? r.x : (e & 3) == 1 ? r.y : (e & 3) == 2 ? r.z : r.w);
+            v[e] = size[e] ? __float_as_uint(score[e]) : 0u;  // similarities are not negative
+        }
+        last = best(v, bv);
+        if (bv == 0) last = best(size, bv);
     }
-    return order;
 }
 
 // Bytes of the class-0 and per-tile matrices the block-sparse path appends
@@ -368,8 +425,6 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
 
     // ---- sketch: the dense product of the lowest values, about
     // kSketchPerSample per sample ----
-    std::vector<u32> order(n), pos(n);
-    for (u64 i = 0; i < n; ++i) order[i] = (u32)i;
     DevBuf d_pos, d_order, d_tile, d_cls_of, d_rowk, jobtab, Wc, kbase;
     const u64 nw_max = mt / 64;
     const u64 nb_max = (T + 1) * nw_max / kScanBlockWords;
@@ -464,6 +519,22 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
     ALLOC(d_cls_of, n * sizeof(u32));
     ALLOC(jobtab, kMaxTiles * sizeof(TcJobDesc));
     CK(cudaMemsetAsync(kbase.p, 0, (T + 1) * sizeof(u64), cs));
+
+    const u64 jstride = round_up(n, 4);  // floats a row of the sketch's similarities
+    auto set_order = [&](const float* d_jf, const u64* d_sz) -> int {
+        static_assert(kMaxTiles * kTile <= 8 * kOrderThreads, "samples per thread");
+        auto k = n <= 4 * kOrderThreads ? k_sample_order<4> : k_sample_order<8>;
+        k<<<1, kOrderThreads, 0, cs>>>(d_jf, (u32)jstride, d_sz, (u32)n, d_order.as<u32>(), d_pos.as<u32>(),
+                                       d_tile.as<u32>(), d_cls_of.as<u32>(), d_rowk.as<u32>());
+        CK(cudaGetLastError());
+        ctx->stats.launches += 1;
+        // the classification's stream reads it (and buffers allocated so far)
+        if (ccs != cs) {
+            CK(cudaEventRecord(slot[0].packed, cs));
+            CK(cudaStreamWaitEvent(ccs, slot[0].packed, 0));
+        }
+        return JSIM_OK;
+    };
 
     // classify the rows of [lo, lo + width) into slot s and scan them; the
     // totals go to the host behind the slot's event
@@ -591,6 +662,19 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
         if (rc) return rc;
         rc = build_batch(ctx, st, sb, lo_s, ws, R_s, stride_s, nullptr, nullptr, nullptr, pb, pe);
         if (rc) return rc;
+        // the rows are known now, by the sketch range's: is the dense call done
+        // before the samples are in order (a tenth aside, for the estimate)?
+        if (may_decline && R_s && !feed) {
+            const double values = (double)std::max<u64>(1, ctx->h_scalars[3]);
+            if (dense_ms((double)R_s * (double)st.N / values) <=
+                0.9 * (order_ms(n) + sparse_ms(0.0))) {
+                declined = true;
+                return JSIM_OK;
+            }
+        }
+        DevBuf Jf;  // the sketch sizes (n u64), then the similarities (n x n floats)
+        u64* d_sz = nullptr;
+        float* d_jf = nullptr;
         if (R_s) {
             DevBuf Cs;
             ALLOC(Cs, n * n * cb);
@@ -598,52 +682,24 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
             const u64 W_s = (R_s + 63) / 64;
             rc = run_product(ctx, choose_variant(ctx, n, W_s), sb.X.as<u64>(), stride_s, n, W_s, Cs.p);
             if (rc) return rc;
-            // the input's validation runs while the host orders the samples
+            // the input's validation runs beside the ordering
             if (sv && !sv->started) {
                 rc = sv->start(ctx, st);
                 if (rc) return rc;
             }
-            // the sizes (n u64) and then the similarities (n x n floats) into
-            // page-locked memory kept by the context: the host only runs the
-            // greedy chain
-            const size_t hb = n * sizeof(u64) + n * n * sizeof(float);
-            if (ctx->h_sketch_bytes < hb) {
-                if (ctx->h_sketch) cudaFreeHost(ctx->h_sketch);
-                ctx->h_sketch = nullptr;
-                ctx->h_sketch_bytes = 0;
-                CK(cudaMallocHost(&ctx->h_sketch, hb));
-                ctx->h_sketch_bytes = hb;
-            }
-            DevBuf Jf;
-            ALLOC(Jf, hb);
+            ALLOC(Jf, round_up(n, 2) * sizeof(u64) + n * jstride * sizeof(float));
             const unsigned g = grid_of(n * n, ctx->sms, 256);
-            u64* d_sz = Jf.as<u64>();
-            float* d_jf = (float*)(d_sz + n);
+            d_sz = Jf.as<u64>();
+            d_jf = (float*)(d_sz + round_up(n, 2));
             if (cb == 8)
-                k_sketch_j<u64><<<g, 256, 0, cs>>>(Cs.as<u64>(), n, d_jf, d_sz);
+                k_sketch_j<u64><<<g, 256, 0, cs>>>(Cs.as<u64>(), n, d_jf, jstride, d_sz);
             else
-                k_sketch_j<u32><<<g, 256, 0, cs>>>(Cs.as<u32>(), n, d_jf, d_sz);
+                k_sketch_j<u32><<<g, 256, 0, cs>>>(Cs.as<u32>(), n, d_jf, jstride, d_sz);
             CK(cudaGetLastError());
             ctx->stats.launches += 1;
-            CK(cudaMemcpyAsync(ctx->h_sketch, Jf.p, hb, cudaMemcpyDeviceToHost, cs));
-            CK(cudaStreamSynchronize(cs));
-            const u64* h_sz = (const u64*)ctx->h_sketch;
-            order = sample_order((const float*)(h_sz + n), h_sz, n);
         }
-        for (u64 k = 0; k < n; ++k) pos[order[k]] = (u32)k;
-        // per plan entry k (the sample at position k): its tile, class and row
-        std::vector<u32> tile(n), cls_of(n), rowk(n);
-        for (u64 k = 0; k < n; ++k) {
-            tile[k] = (u32)(k / kTile);
-            cls_of[k] = 1 + tile[k];
-            rowk[k] = (u32)k;
-        }
-        CK(cudaMemcpyAsync(d_pos.p, pos.data(), n * sizeof(u32), cudaMemcpyHostToDevice, cs));
-        CK(cudaMemcpyAsync(d_order.p, order.data(), n * sizeof(u32), cudaMemcpyHostToDevice, cs));
-        CK(cudaMemcpyAsync(d_tile.p, tile.data(), n * sizeof(u32), cudaMemcpyHostToDevice, cs));
-        CK(cudaMemcpyAsync(d_cls_of.p, cls_of.data(), n * sizeof(u32), cudaMemcpyHostToDevice, cs));
-        CK(cudaMemcpyAsync(d_rowk.p, rowk.data(), n * sizeof(u32), cudaMemcpyHostToDevice, cs));
-        CK(cudaStreamSynchronize(cs));  // the host vectors are released at return
+        rc = set_order(d_jf, d_sz);
+        if (rc) return rc;
 
         if (may_decline && R_s) {
             // the sketch range's rows by class: is the product at least halved?
@@ -675,9 +731,8 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
             }
         }
     } else {
-        for (u64 k = 0; k < n; ++k) pos[k] = (u32)k;
-        CK(cudaMemcpyAsync(d_pos.p, pos.data(), n * sizeof(u32), cudaMemcpyHostToDevice, cs));
-        CK(cudaStreamSynchronize(cs));
+        const int rc = set_order(nullptr, nullptr);
+        if (rc) return rc;
     }
     ctx->stats.variant = JSIM_VARIANT_SPARSE;
 
