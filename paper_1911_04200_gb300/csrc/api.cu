@@ -250,7 +250,7 @@ int all_pairs_impl(jsim_ctx* ctx, const jsim_sets* sets, void* C, uint64_t* size
     u64 feed_mt = 0, fminid = 0, fmaxid = 0;
     const u64* hv = nullptr;
     if (sparse && feed_applies(ctx, sets, hoff, fminid, fmaxid, hv) &&
-        (feed_mt = sparse_batch_rows(ctx, n, fmaxid - fminid)) != 0 && fmaxid / feed_mt - fminid / feed_mt >= 3) {
+        (feed_mt = feed_batch_rows(ctx, n, hoff[n], fmaxid - fminid)) != 0 && fmaxid / feed_mt - fminid / feed_mt >= 3) {
         // page-locked host input: copied piece by piece under the batch loop
         rc = stage_input(ctx, sets, st, hoff, false);
         if (rc) return rc;

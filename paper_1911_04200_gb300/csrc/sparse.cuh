@@ -326,6 +326,17 @@ u64 sparse_batch_rows(const jsim_ctx* ctx, u64 n, u64 span, bool windowed = fals
     return std::max(mt, kMinClassRows);
 }
 
+// Batch width of page-locked input fed in pieces (0: as sparse_batch_rows).
+// The ranked ingest takes wide batches; eight of them or more keep the first
+// piece's copy and the last piece's ingest short.
+u64 feed_batch_rows(const jsim_ctx* ctx, u64 n, u64 N, u64 span)
+{
+    if (ctx->opt.batch_rows || N > kRankMaxValues) return sparse_batch_rows(ctx, n, span);
+    u64 mt = std::max(kMinClassRows, auto_batch_rows(span + 1 ? span + 1 : ~0ull));
+    while (mt > kMinClassRows && span / mt < 8) mt >>= 1;
+    return mt;
+}
+
 // The block-sparse path of jsim_all_pairs: JSIM_ERR_UNSUPPORTED where it does
 // not apply (more than kMaxTiles tiles, no tensor cores, a batch width that
 // is not a multiple of kMinClassRows); with may_decline, declined = true
@@ -350,11 +361,12 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
     const u64 span = st.N ? st.maxid - st.minid : 0;
     // Windowed ingest where the values are dense enough for windows of
     // 2^wl rows, on device-resident input (the per-value ingest otherwise).
-    // Input fed piece by piece keeps the per-value ingest: the windowed
-    // kernels hold an SM's registers for tens of microseconds per CTA, which
-    // holds back the copy CTAs that feed the link (measured on the default
-    // workload from page-locked host memory: 70 to 75 ms per call windowed,
-    // 67.5 ms per value).
+    // Input fed piece by piece is not windowed: the windowed kernels hold an
+    // SM's registers for tens of microseconds per CTA, which holds back the
+    // copy CTAs that feed the link (1.3e9 values from page-locked host memory:
+    // 70 to 75 ms per call windowed, 67.5 ms per value).  It takes the ranked
+    // ingest, a piece's batches beside the next pieces' copies (2.1e8 values:
+    // 16.5 ms per value in 2^27-row batches, 12.3 ranked; the link alone 9.7).
     const int wl = kWinLog;
     const double per_window =
         st.N ? (double)st.N / (double)n / ((double)span + 1.0) * (double)(1ull << wl) : 0.0;
@@ -368,7 +380,7 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
     const u64 dense_mt = st.N ? dense_batch_rows(ctx, n, st.N, st.minid, st.maxid, &dense_ingest) : 0;
     const double windowed_ms = ((double)span + 1.0) / 4294967296.0 * (double)T * kWinTileMs[twice] +
                                (double)st.N * kWinValueMs[twice];
-    bool windowed = false, ranked = !feed && st.N && st.N <= kRankMaxValues && !ctx->opt.batch_rows;
+    bool windowed = false, ranked = st.N && st.N <= kRankMaxValues && !ctx->opt.batch_rows;
     u64 mt = 0;
     double sparse_ingest = 0;
     auto choose_ingest = [&]() {
@@ -376,7 +388,9 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
         if (ranked && windowed && (per_window >= kWinSureValues || windowed_ms <= dense_ingest)) ranked = false;
         if (ranked) windowed = false;
         mt = feed ? feed->mt : ranked ? std::max(kMinClassRows, dense_mt) : sparse_batch_rows(ctx, n, span, windowed);
-        sparse_ingest = ranked     ? dense_ingest
+        sparse_ingest = ranked     ? (feed ? (double)(st.maxid / mt - st.minid / mt + 1) * kDenseBatchMs +
+                                                (double)st.N * kDenseValueMs[twice][0]
+                                          : dense_ingest)
                         : windowed ? windowed_ms
                         : mt       ? (double)(st.maxid / mt - st.minid / mt + 1) * kPerBatchMs[twice] +
                                    (double)st.N * kPerValueMs
