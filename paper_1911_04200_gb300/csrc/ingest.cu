@@ -7,10 +7,80 @@ namespace jsim {
 
 namespace {
 
+// Every sample's first value at or above lo and at or above hi (hi == 0: its
+// end) into the plan, and the smallest value after the batch into *s_next.
+// G lanes search one sample: a step probes G places of each of its two ranges,
+// and a thread has U samples under way, so the chain of dependent loads is
+// short: 50,000 values take 4 steps for 64 samples (G = 16), 16 for 1024
+// (G = 1), where a bisection per end takes 32.  (On unsorted values, any place
+// of the range.)
+template <int U>
+__device__ __forceinline__ void plan_search(const u64* __restrict__ offsets, const u64* __restrict__ ids, u64 n, u64 lo,
+                                            u64 hi, const Plan& plan, const u32* __restrict__ perm,
+                                            const u64* __restrict__ ends, u32 G, u64* s_next, int* s_has_next)
+{
+    const u32 lane = threadIdx.x & 31, gl = lane & (G - 1), g0 = lane - gl;
+    const u32 gmask = G == 32 ? 0xffffffffu : (1u << G) - 1u;
+    const u64 groups = kPlanThreads / G, group = threadIdx.x / G;
+    for (u64 j0 = 0; j0 < n; j0 += (u64)U * groups) {
+        u64 end[U], a[2 * U], b[2 * U];  // a, b: what is left of each range
+        #pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const u64 j = j0 + (u64)u * groups + group;
+            end[u] = a[2 * u] = 0;
+            if (j < n) {
+                const u64 sj = perm ? (u64)perm[j] : j;
+                a[2 * u] = offsets[sj];
+                end[u] = ends ? ends[sj] : offsets[sj + 1];
+            }
+            a[2 * u + 1] = hi ? a[2 * u] : end[u];
+            b[2 * u] = b[2 * u + 1] = end[u];
+        }
+        // (every step at least halves what is left of a range)
+        for (int round = 0; round < 65; ++round) {
+            bool left = false;
+            #pragma unroll
+            for (int k = 0; k < 2 * U; ++k) left = left || a[k] < b[k];
+            if (!__any_sync(0xffffffffu, left)) break;
+            u64 x[2 * U], step[2 * U];
+            bool in[2 * U];
+            #pragma unroll
+            for (int k = 0; k < 2 * U; ++k) {
+                const u64 len = b[k] - a[k];
+                step[k] = len <= G ? 1 : (len >> 32) ? len / (G + 1) + 1 : (u64)((u32)len / (G + 1)) + 1;
+                const u64 p = a[k] + (gl + 1) * step[k] - 1;
+                in[k] = p < b[k];
+                x[k] = in[k] ? ids[p] : 0ull;
+            }
+            #pragma unroll
+            for (int k = 0; k < 2 * U; ++k) {
+                const u32 m = __ballot_sync(0xffffffffu, in[k] && x[k] < ((k & 1) ? hi : lo));
+                const u32 below = (u32)__popc((m >> g0) & gmask);
+                a[k] += below * step[k];
+                const u64 top = a[k] + step[k] - 1;  // the first probe not below
+                if (below < G && top < b[k]) b[k] = top;
+            }
+        }
+        #pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const u64 j = j0 + (u64)u * groups + group;
+            if (j >= n || gl != 0) continue;
+            const u64 q = max(a[2 * u], a[2 * u + 1]);
+            plan.beg[j] = a[2 * u];
+            plan.len[j] = q - a[2 * u];
+            if (q < end[u]) {
+                atomicMin((unsigned long long*)s_next, (unsigned long long)ids[q]);
+                *s_has_next = 1;
+            }
+        }
+    }
+}
+
 // One CTA: per-sample [beg, beg+len) of values in [lo, hi) and chunk prefix.
 // With perm, entry i of the plan is sample perm[i] (the ingest kernels then
 // walk the samples in that order).  With ends, sample i is searched in
-// [offsets[i], ends[i]) only.
+// [offsets[i], ends[i]) only.  Bound by the searches' dependent loads: 64
+// samples of 50,000 values 24.6 us by bisection, 9 us here.
 __global__ void __launch_bounds__(kPlanThreads)
 k_plan(const u64* __restrict__ offsets, const u64* __restrict__ ids, u64 n, u64 lo, u64 hi,
        int full, Plan plan, const u32* __restrict__ perm, const u64* __restrict__ ends)
@@ -20,27 +90,31 @@ k_plan(const u64* __restrict__ offsets, const u64* __restrict__ ids, u64 n, u64 
     __shared__ int s_has_next;
     if (threadIdx.x == 0) { s_next = ~0ull; s_has_next = 0; }
     __syncthreads();
+    if (!full) {
+        u32 G = 1;
+        while (G < 32 && 2 * (u64)G * n <= kPlanThreads) G *= 2;
+        if (n <= kPlanThreads)
+            plan_search<1>(offsets, ids, n, lo, hi, plan, perm, ends, G, &s_next, &s_has_next);
+        else
+            plan_search<2>(offsets, ids, n, lo, hi, plan, perm, ends, G, &s_next, &s_has_next);
+        __syncthreads();
+    }
     u64 carry = 0, total_len = 0;
     for (u64 base = 0; base < n; base += kPlanThreads) {
-        u64 i = base + threadIdx.x;
-        u64 b = 0, l = 0, nch = 0;
+        const u64 i = base + threadIdx.x;
+        u64 l = 0;
         if (i < n) {
-            const u64 si = perm ? (u64)perm[i] : i;
-            u64 s = offsets[si], e = ends ? ends[si] : offsets[si + 1];
-            if (!full) {
-                const u64 se = e;
-                u64 bb = lower_bound_u64(ids, s, e, lo);
-                u64 ee = hi == 0 ? e : lower_bound_u64(ids, bb, e, hi);  // hi==0: unbounded
-                s = bb; e = ee;
-                if (ee < se) {  // first value of this sample after the batch
-                    atomicMin(&s_next, ids[ee]);
-                    s_has_next = 1;
-                }
+            if (full) {
+                const u64 si = perm ? (u64)perm[i] : i;
+                const u64 s = offsets[si];
+                l = (ends ? ends[si] : offsets[si + 1]) - s;
+                plan.beg[i] = s;
+                plan.len[i] = l;
+            } else {
+                l = plan.len[i];
             }
-            b = s; l = e - s; nch = (l + kChunk - 1) / kChunk;
-            plan.beg[i] = b;
-            plan.len[i] = l;
         }
+        const u64 nch = (l + kChunk - 1) / kChunk;
         u64 ex;
         u64 tot = block_exclusive_scan<kPlanThreads>(nch, ex, sm);
         if (i < n) plan.cofs[i] = carry + ex;

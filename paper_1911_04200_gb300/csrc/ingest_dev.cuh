@@ -93,21 +93,32 @@ __device__ __forceinline__ void fetch_chunk(const Plan& plan, u64 n, u64 nch, in
     }
 }
 
-// Inclusive OR over the lanes that share key q, accumulated toward the
-// segment's first lane (q is non-decreasing across lanes).  Returns true on
-// the lane that must publish the segment's value.
+// OR of v over every run of neighbouring lanes with the same key q, left on
+// the run's first lane.  Returns true on that lane, which publishes it.  (Of
+// keys that come back after others only neighbours combine, so what is
+// published is complete as long as it is OR-ed into its place.)
+//
+// The keys are compared once, with the lane before; the runs' ends follow from
+// one ballot, and a step is one shuffle of v, as many as the longest run takes:
+// none for values in words of their own, five for a run of a whole warp.
+// (Pack of 1.7e8 values, rows of 42 of them a word apart: 1.64 -> 1.43 ms
+// against comparing the keys at every step.)
 template <typename T>
 __device__ __forceinline__ bool segmented_or(u64 q, T& v)
 {
-    const int lane = threadIdx.x & 31;
-    #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        T w = __shfl_down_sync(0xffffffffu, v, o);
-        u64 qq = __shfl_down_sync(0xffffffffu, q, o);
-        if (lane + o < 32 && qq == q) v |= w;
+    const u32 lane = threadIdx.x & 31;
+    const u64 before = __shfl_up_sync(0xffffffffu, q, 1);  // every lane takes part
+    const bool head = lane == 0 || before != q;
+    const u32 heads = __ballot_sync(0xffffffffu, head);
+    if (heads == 0xffffffffu) return true;
+    const u32 above = heads & ~(0xffffffffu >> (31 - lane));  // heads of the runs after this lane's
+    const u32 left = above ? (u32)__ffs((int)above) - 1 - lane : 32 - lane;  // lanes to the end of the run
+    const u32 longest = __reduce_max_sync(0xffffffffu, left);
+    for (u32 o = 1; o < longest; o <<= 1) {
+        const T w = __shfl_down_sync(0xffffffffu, v, o);
+        if (o < left) v |= w;
     }
-    u64 qprev = __shfl_up_sync(0xffffffffu, q, 1);
-    return lane == 0 || qprev != q;
+    return head;
 }
 
 }  // namespace
