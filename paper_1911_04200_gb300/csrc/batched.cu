@@ -39,6 +39,10 @@ struct Col {
 // finished on kLanes side streams at once: their kernels are small, and one
 // stream would run them one after another.
 constexpr int kLanes = 4;
+// What a batch costs a lane whatever it holds, the lanes running beside one
+// another.  20 collections of 8 to 512 samples x 20,000 values in [0, 2^32),
+// the 13 below 256 sharing launches: 7.5 ms in 2^29-row batches, 6.8 in 2^30.
+constexpr double kWaveBatchMs = 0.06;
 
 // Everything one wave of collections needs on the device; kept alive by the
 // graph cache so a replay finds the same addresses.
@@ -50,7 +54,7 @@ struct Wave {
     DevBuf bitmap[kLanes], seen[kLanes], dir[kLanes], bsum[kLanes], boff[kLanes], R[kLanes];
     DevBuf jobtab;          // tensor-core job table
     DevBuf cstage, jstage;  // host-output staging
-    u64 max_mt = 0;
+    u64 max_mt = 0, batches = 0;
     int variant = JSIM_VARIANT_TC;
     int word_bits = 64;
     int tile_n = 256;       // tensor-core tile width (128 x tile_n tiles)
@@ -432,34 +436,44 @@ replan:
     }
 
     // ---- batch plan and packed-matrix bound of every collection ----
+    // A lane's batch costs kWaveBatchMs whatever it holds: few values take
+    // wide batches, as in the plain call (dense_batch_rows), as far as the
+    // lanes' bitmaps stay within what the packed matrices take (a call's
+    // scratch at most doubles).
     size_t x_tot = 0, c_tot = 0, cs_tot = 0, js_tot = 0;
-    for (auto& x : w.cols) {
-        x.empty = x.N == 0;
-        const u64 span = x.empty ? 0 : x.maxid - x.minid;
-        // batches of up to 2^29 rows (a 64 MiB filter bitmap): fewer, longer
-        // batches than the plain call's 2^28, since a batched call pays per
-        // batch launches for many small collections.  Measured on 200
-        // collections spanning [0, 2^32) (ms per call, rows per batch 2^26 /
-        // 2^28 / 2^29 / 2^30 / 2^31 / 2^32): 385 / 247 / 234 / 237 / 254 / 272
-        u64 one = 64;
-        while (one < span + 1 && one < (1ull << 29)) one <<= 1;
-        x.mt = ctx->opt.batch_rows ? ctx->opt.batch_rows : one;
-        x.lo0 = x.empty ? 0 : x.minid / x.mt * x.mt;
-        x.rounds = x.empty ? 0 : x.maxid / x.mt - x.minid / x.mt + 1;
-        if (x.rounds > 4096) return JSIM_ERR_UNSUPPORTED;  // value span too wide for one batched plan
-        // sum_l ceil(R_l / 64) <= N / 64 + rounds
-        x.stride = round_up(x.N / 64 + x.rounds + 1, kWordPad);
-        x.n_pad = round_up(std::max<u64>(x.n, 1), kRowPad);
-        x.x_off = x_tot;
-        x_tot += x.n_pad * x.stride;
-        x.c_off = c_tot;
-        c_tot += x.n * x.n * cb;
-        cs_tot += x.n * x.n * cb;
-        js_tot += x.n * x.n * sizeof(double);
-        w.max_mt = std::max(w.max_mt, x.mt);
-        ctx->stats.batches += x.rounds;
-    }
-    {
+    auto plan_wave = [&](u64 widest) -> int {
+        x_tot = c_tot = cs_tot = js_tot = 0;
+        w.max_mt = 0;
+        u64 batches = 0;
+        for (auto& x : w.cols) {
+            x.empty = x.N == 0;
+            const u64 span = x.empty ? 0 : x.maxid - x.minid;
+            u64 one = 64;
+            while (one < span + 1 && one < (1ull << 29)) one <<= 1;
+            x.mt = ctx->opt.batch_rows ? ctx->opt.batch_rows : one;
+            if (!x.empty && x.maxid / x.mt - x.minid / x.mt + 1 > 4096)
+                return JSIM_ERR_UNSUPPORTED;  // value span too wide for one batched plan
+            if (widest > x.mt && !x.empty && !ctx->opt.batch_rows)
+                x.mt = std::max(x.mt, std::min(widest, dense_batch_rows(ctx, x.n, x.N, x.minid, x.maxid, nullptr,
+                                                                        kWaveBatchMs, kLanes)));
+            x.lo0 = x.empty ? 0 : x.minid / x.mt * x.mt;
+            x.rounds = x.empty ? 0 : x.maxid / x.mt - x.minid / x.mt + 1;
+            // sum_l ceil(R_l / 64) <= N / 64 + rounds
+            x.stride = round_up(x.N / 64 + x.rounds + 1, kWordPad);
+            x.n_pad = round_up(std::max<u64>(x.n, 1), kRowPad);
+            x.x_off = x_tot;
+            x_tot += x.n_pad * x.stride;
+            x.c_off = c_tot;
+            c_tot += x.n * x.n * cb;
+            cs_tot += x.n * x.n * cb;
+            js_tot += x.n * x.n * sizeof(double);
+            w.max_mt = std::max(w.max_mt, x.mt);
+            batches += x.rounds;
+        }
+        w.batches = batches;
+        return JSIM_OK;
+    };
+    auto alloc_lanes = [&]() -> int {
         const u64 nwords = std::max<u64>(w.max_mt / 64, 1);
         const u64 nb = (nwords + kScanBlockWords - 1) / kScanBlockWords;
         for (int l = 0; l < kLanes; ++l) {
@@ -470,6 +484,28 @@ replan:
             ALLOC(w.boff[l], std::max<u64>(nb, 1) * 8);
             ALLOC(w.R[l], 8);
         }
+        return JSIM_OK;
+    };
+    {
+        const u64 narrow = 1ull << 29;
+        int rc = plan_wave(narrow);
+        if (rc) return rc;
+        u64 widest = narrow;
+        const double bits = ctx->opt.filter_min == 2 ? 2.5 : 1.5;  // bitmap, directory (and every row's bitmap)
+        while (widest < (1ull << 32) && kLanes * bits * (double)(2 * widest) / 8.0 <= 8.0 * (double)x_tot) widest *= 2;
+        if (widest > narrow) {
+            rc = plan_wave(widest);
+            if (rc) return rc;
+        }
+        rc = alloc_lanes();
+        if (rc == JSIM_ERR_OOM && w.max_mt > narrow && !ctx->opt.batch_rows) {  // no room for the wide batches
+            for (int l = 0; l < kLanes; ++l)
+                for (DevBuf* d : {&w.bitmap[l], &w.seen[l], &w.dir[l], &w.bsum[l], &w.boff[l]}) d->release();
+            rc = plan_wave(narrow);
+            if (!rc) rc = alloc_lanes();
+        }
+        if (rc) return rc;
+        ctx->stats.batches += w.batches;
         ALLOC(w.xpool, std::max<size_t>(x_tot, 1) * 8);
         ALLOC(w.cpool, std::max<size_t>(c_tot, 8));
         ALLOC(w.scal, 2 * sizeof(u64) * k);

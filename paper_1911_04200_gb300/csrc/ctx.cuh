@@ -489,12 +489,15 @@ u64 auto_batch_rows(u64 domain)
 constexpr double kDenseBatchMs = 0.17;
 constexpr double kDenseValueMs[2][5] = {{2.8e-8, 3.4e-8, 5.0e-8, 7.0e-8, 8.2e-8},   // one filter
                                         {2.8e-8, 3.9e-8, 6.1e-8, 8.2e-8, 9.8e-8}};  // two-or-more
-u64 dense_batch_rows(const jsim_ctx* ctx, u64 n, u64 N, u64 minid, u64 maxid, double* ms = nullptr)
+// (batch_ms: kDenseBatchMs, or what else a batch costs the caller; copies: how
+// many sets of bitmaps it keeps)
+u64 dense_batch_rows(const jsim_ctx* ctx, u64 n, u64 N, u64 minid, u64 maxid, double* ms = nullptr,
+                     double batch_ms = kDenseBatchMs, int copies = 1)
 {
     const u64 span = maxid - minid;
     const double* value_ms = kDenseValueMs[ctx->opt.filter_min == 2];
     auto cost = [&](u64 w, int k) {
-        return (double)(maxid / w - minid / w + 1) * kDenseBatchMs + (double)N * value_ms[k];
+        return (double)(maxid / w - minid / w + 1) * batch_ms + (double)N * value_ms[k];
     };
     u64 best = ctx->opt.batch_rows ? ctx->opt.batch_rows : auto_batch_rows(span + 1 ? span + 1 : ~0ull);
     double best_ms = cost(best, 0);
@@ -506,7 +509,7 @@ u64 dense_batch_rows(const jsim_ctx* ctx, u64 n, u64 N, u64 minid, u64 maxid, do
         if (t >= best_ms) continue;
         const double held = std::min(1.0, (double)w / ((double)span + 1.0)) * (double)N;
         const double x_bytes = (double)round_up(std::max<u64>(n, 1), kRowPad) * held / 8.0;
-        const double bytes = x_bytes + (double)w / 8.0 * (ctx->opt.filter_min == 2 ? 2.5 : 1.5);
+        const double bytes = x_bytes + copies * (double)w / 8.0 * (ctx->opt.filter_min == 2 ? 2.5 : 1.5);
         if (!total_b && cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) { cudaGetLastError(); break; }
         if (x_bytes > (double)(4ull << 30) || bytes > (double)free_b / 4.0) continue;
         best = w;
