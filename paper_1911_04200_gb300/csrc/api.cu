@@ -510,7 +510,8 @@ int jsim_product(jsim_ctx* ctx, const uint64_t* words, uint64_t n, uint64_t W, u
     DevBuf Cacc;
     ALLOC(Cacc, n * n * cb);
     CK(cudaMemsetAsync(Cacc.p, 0, n * n * cb, ctx->stream));
-    int v = variant == JSIM_VARIANT_AUTO ? choose_variant(ctx, n, W) : variant;
+    const bool aligned = (uintptr_t)words % 16 == 0 && stride % 2 == 0;
+    int v = variant == JSIM_VARIANT_AUTO ? choose_variant(ctx, n, W, aligned) : variant;
     CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(u32), ctx->stream));
     DevBuf useful;
     if (W) {
@@ -636,7 +637,8 @@ extern "C" int jsim_product_noalloc(jsim_ctx* ctx, const uint64_t* words, uint64
     u32* err = (u32*)(scratch + kNoAllocCountBytes);
     CK(cudaMemsetAsync(scratch, 0, (size_t)(n * n) * cb, ctx->stream));
     CK(cudaMemsetAsync(err, 0, sizeof(u32), ctx->stream));
-    const int v = variant == JSIM_VARIANT_AUTO ? choose_variant(ctx, n, W) : variant;
+    const bool aligned = (uintptr_t)words % 16 == 0 && stride % 2 == 0;
+    const int v = variant == JSIM_VARIANT_AUTO ? choose_variant(ctx, n, W, aligned) : variant;
     if (W) {
         int rc = run_product(ctx, v, (const u64*)words, stride, n, W, scratch, err);
         if (rc) return rc;

@@ -519,18 +519,20 @@ u64 dense_batch_rows(const jsim_ctx* ctx, u64 n, u64 N, u64 minid, u64 maxid, do
     return best;
 }
 
-// Variant choice, from a sweep on GB300 (random packed words, Tbit-ops/s):
-//   n      64    128   192   256   512   1024  2048
-//   POPC   71    92    104   111   123   130   142
-//   TC     32    124   193   333   491   654   831
-//   TC2    24    95    211   377   601   848   1069
-// (the legacy mma.sync kernels stay at or below POPC).  Tensor tiles of 128
-// or 256 samples are mostly idle for small n.
-int choose_variant(jsim_ctx* ctx, u64 n, u64 W)
+// Variant choice, from products alone on GB300 (us per call, of which 55 are
+// the call itself; random words):
+//   n x words     64 x 512  64 x 65,536  128 x 4096  128 x 65,536  160 x 4096  160 x 65,536
+//   POPC            86        185          84          434           120         815
+//   TC              59         96          86          111            95         324
+//   TC2             70        134          71          134            71         134
+// TC up to 128 samples is one 128 x 128 tile (the diagonal-tile kernel), above
+// it a padded one; it loads words by TMA, and rows that are not 16-byte
+// aligned take the byte-operand kernel, half as fast as POPC up to 96 samples.
+int choose_variant(jsim_ctx* ctx, u64 n, u64 W, bool aligned = true)
 {
     (void)W;
-    if (n <= 96 || !product_tc_supported(ctx->opt.device)) return JSIM_VARIANT_POPC;
-    return n <= 160 ? JSIM_VARIANT_TC : JSIM_VARIANT_TC2;
+    if (!product_tc_supported(ctx->opt.device) || (n <= 96 && !aligned)) return JSIM_VARIANT_POPC;
+    return n <= 128 ? JSIM_VARIANT_TC : JSIM_VARIANT_TC2;
 }
 
 // The semiring product C += X X^T with the chosen variant; err is the device

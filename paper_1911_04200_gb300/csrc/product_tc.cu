@@ -573,6 +573,13 @@ bool product_tc_supported(int device)
 
 cudaError_t product_tc(ProductArgs& a, cudaStream_t st)
 {
+    // one 128 x 128 tile: the diagonal-tile kernel (16-byte aligned rows)
+    if (a.n && a.n <= (u64)tcs::kM && a.W) {
+        const TcJobDesc job{a.X, nullptr, a.C, a.stride, a.n, a.W, a.ldc};
+        bool taken = false;
+        const cudaError_t e = product_tc_diag(&job, 1, a.count_bits, a.sms, a.err, a.timeout_ms, st, &a.launches, &taken);
+        if (e != cudaSuccess || taken) return e;
+    }
     return product_tc_single(a, st);
 }
 
