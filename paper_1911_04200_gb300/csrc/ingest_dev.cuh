@@ -103,11 +103,11 @@ __device__ __forceinline__ void fetch_chunk(const Plan& plan, u64 n, u64 nch, in
 // none for values in words of their own, five for a run of a whole warp.
 // (Pack of 1.7e8 values, rows of 42 of them a word apart: 1.64 -> 1.43 ms
 // against comparing the keys at every step.)
-template <typename T>
-__device__ __forceinline__ bool segmented_or(u64 q, T& v)
+template <typename T, typename K>
+__device__ __forceinline__ bool segmented_or(K q, T& v)
 {
     const u32 lane = threadIdx.x & 31;
-    const u64 before = __shfl_up_sync(0xffffffffu, q, 1);  // every lane takes part
+    const K before = __shfl_up_sync(0xffffffffu, q, 1);  // every lane takes part
     const bool head = lane == 0 || before != q;
     const u32 heads = __ballot_sync(0xffffffffu, head);
     if (heads == 0xffffffffu) return true;
