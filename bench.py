@@ -260,11 +260,13 @@ def roofline_for(variant, bitops_per_launch, ms_per_launch, peaks, traffic):
         return {"bound": "tensor", "achieved": round(achieved_t, 3), "peak": peak, "unit": "Tbit-ops/s",
                 "frac": round(achieved_t / peak, 4), "traffic": traffic,
                 "peak_source": "measured legacy mma.sync s8/b1 issue rate (%.0f T ops/s)" % peak}
+    # (the SM-pair and diagonal-tile products multiply 4-bit operands: x 6)
+    kind, ratio = ("fp4", 6.0) if variant in ("tc2", "sparse") else ("fp8", 2.0)
     flops = 2.0 * achieved_t
-    peak = pk.get("bf16_tflops_sustained", 1700.0) * 2.0
+    peak = pk.get("bf16_tflops_sustained", 1700.0) * ratio
     return {"bound": "tensor", "achieved": round(flops, 2), "peak": round(peak, 1), "unit": "TFLOP/s",
             "frac": round(flops / peak, 4), "traffic": traffic,
-            "peak_source": "%s bf16 sustained x 2 (fp8:bf16 nominal ratio)" % src}
+            "peak_source": "%s bf16 sustained x %d (%s:bf16 nominal ratio)" % (src, int(ratio), kind)}
 
 
 def traffic_from_profiles(variant, workload):

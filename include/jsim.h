@@ -78,8 +78,9 @@ extern "C" {
 #define JSIM_VARIANT_B1   2  /* legacy tensor mma.sync .b1 with .and.popc */
 #define JSIM_VARIANT_I8   3  /* legacy tensor mma.sync .s8, bits unpacked to 0/1 bytes, s32 accumulate */
 #define JSIM_VARIANT_F8   4  /* legacy tensor mma.sync .e4m3, bits unpacked to 0/1.0, f32 accumulate in exact ranges */
-#define JSIM_VARIANT_TC   5  /* tcgen05.mma kind::f8f6f4 with TMEM accumulators, 0/1.0 e4m3 operands */
-#define JSIM_VARIANT_TC2  6  /* as TC, on pairs of SMs (cta_group::2, 256 x 256 tiles) */
+#define JSIM_VARIANT_TC   5  /* tcgen05.mma with TMEM accumulators: one 128 x 128 tile of 4-bit 0/1 operands up to 128
+                                samples (16-byte aligned rows), else kind::f8f6f4, 0/1.0 e4m3 operands */
+#define JSIM_VARIANT_TC2  6  /* tcgen05.mma kind::mxf4 on pairs of SMs (cta_group::2, 256 x 256 tiles) */
 #define JSIM_VARIANT_SPARSE 7 /* block-sparse (jsim_all_pairs only, 1..2048 samples, tensor cores):
                                 samples ordered by a sketch of their similarity into tiles of
                                 128, rows held by one tile multiplied within that tile's
@@ -172,7 +173,7 @@ typedef struct {
     uint64_t h2d_pieces;       /* page-locked host input read by the device in this many value-range
                                   pieces while the batch loop ran (0: not fed in pieces) */
     uint64_t windows;          /* row windows the block-sparse variant's windowed ingest classified and
-                                  packed (0: its per-value ingest ran, or another variant) */
+                                  packed (0: its ranked or per-value ingest ran, or another variant) */
 } jsim_stats;
 
 /* Fill *opt with the defaults described above. */

@@ -15,7 +15,8 @@
 //     similar to any sample already in the current tile of 128), so that
 //     samples sharing many values land in the same tile.
 //  2. Row classes.  Per row batch, every tile of 128 samples (in that order)
-//     gets its own filter bitmap (Eq. 5 restricted to the tile's samples).
+//     gets its own filter bitmap (Eq. 5 restricted to the tile's samples), over
+//     the batch's values or, on thin ranges, over its numbered nonzero rows.
 //     A row held by two or more tiles is of class 0; a row held by tile t
 //     alone is of class 1 + t.  Every class is rank-scanned (Eq. 6), so the
 //     packed matrix of the batch splits into a class-0 matrix (all samples)
@@ -24,7 +25,7 @@
 //     Class 1 + t words: a 128 x 128 product of tile t only, added to the
 //     diagonal block of tile t - the only block they can change, since no
 //     other sample holds those rows.  All tiles' blocks run in one launch of
-//     the job-table product.  The words of successive batches are appended
+//     the diagonal-tile product.  The words of successive batches are appended
 //     (Eq. 4) and multiplied when the matrices fill and at the end.  C
 //     accumulates in sample-order positions; the epilogue reads it back
 //     through the order.
