@@ -164,7 +164,7 @@ typedef struct {
                                   the upper triangle they multiplied): bitops_dense, except for the
                                   block-sparse variant, which skips the blocks no row reaches */
     uint64_t tile_n;           /* a batched call's tensor-core tiles: 128 x tile_n (256 or 128, as
-                                  tuned); 0 when its product ran on CUDA cores */
+                                  tuned); 0 when its product ran otherwise */
     uint64_t pack_bytes;       /* bytes the pack kernels read and wrote by algorithm: 8 per value
                                   packed plus 8 per word of the packed matrices they fill (zero
                                   words included) */

@@ -16,9 +16,9 @@
 //   * with device-resident inputs and outputs, the whole launch sequence is
 //     captured once into a CUDA graph and replayed by later calls on the same
 //     collections.
-// An autotuner times the candidate products (tcgen05, CUDA-core with 64-bit
-// and 32-bit words) on the first call of a collection shape and keeps the
-// fastest for that shape.
+// An autotuner times the candidate products (tcgen05 on SM pairs and diagonal
+// tiles, tcgen05 over the table, CUDA-core with 64-bit and 32-bit words) on the
+// first call of a collection shape and keeps the fastest for that shape.
 #include <algorithm>
 #include "ctx.cuh"
 
@@ -142,6 +142,32 @@ int enqueue_wave(jsim_ctx* ctx, Wave& w, void* const* C, double* const* J, bool 
                                         ctx->sms, ctx->d_err, ctx->opt.timeout_ms > 0 ? ctx->opt.timeout_ms : 2000,
                                         st, &launches, tile_n);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "batched tcgen05 product");
+        ctx->stats.product_launches += launches;
+        ctx->stats.launches += launches;
+    } else if (variant == JSIM_VARIANT_TC2) {
+        // 4-bit operands: collections of one tile together, the others one by one
+        const int to = ctx->opt.timeout_ms > 0 ? ctx->opt.timeout_ms : 2000;
+        std::vector<TcJobDesc> small;
+        for (TcJobDesc& j : wave_jobs(w)) {
+            if (j.n <= 128) {
+                j.W = j.stride;
+                small.push_back(j);
+                continue;
+            }
+            ProductArgs a{};
+            a.X = j.X; a.stride = j.stride; a.n = j.n; a.W = j.stride; a.Wdev = j.Wdev; a.C = j.C; a.ldc = j.ldc;
+            a.count_bits = ctx->opt.count_bits; a.sms = ctx->sms; a.timeout_ms = to; a.err = ctx->d_err;
+            cudaError_t e = product_tc_pair(a, st);
+            if (e != cudaSuccess) return cuda_fail(ctx, e, "batched SM-pair product");
+            ctx->stats.product_launches += a.launches;
+            ctx->stats.launches += a.launches;
+        }
+        int launches = 0;
+        bool taken = true;
+        if (!small.empty())
+            CK(product_tc_diag(small.data(), (int)small.size(), ctx->opt.count_bits, ctx->sms, ctx->d_err, to, st,
+                               &launches, &taken));
+        if (!taken) return JSIM_ERR_UNSUPPORTED;  // (only a candidate where the rows are aligned)
         ctx->stats.product_launches += launches;
         ctx->stats.launches += launches;
     } else {
@@ -551,6 +577,10 @@ replan:
         // their rows once), CUDA-core products on 64- and 32-bit words
         std::vector<jsim_tuned> cands;
         if (tc_ok) {
+            static_assert(kWordPad % 2 == 0, "16-byte aligned rows");
+            // 4-bit operands (13 collections of 31 to 231 samples x 20,000 values,
+            // whole call: 6.8 ms with byte tiles, 6.1)
+            if (!ctx->opt.tile_n && (uintptr_t)w.xpool.p % 16 == 0) cands.push_back({JSIM_VARIANT_TC2, 64, 256});
             if (ctx->opt.tile_n != 128) cands.push_back({JSIM_VARIANT_TC, 64, 256});
             if (ctx->opt.tile_n != 256) cands.push_back({JSIM_VARIANT_TC, 64, 128});
         }

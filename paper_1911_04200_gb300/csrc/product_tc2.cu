@@ -354,9 +354,10 @@ struct Accum {
 // otherwise the unpacking warps copy their rows 8 bytes at a time.
 template <typename CT, bool TMA>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-k_prod_tc2(const __grid_constant__ CUtensorMap map, const u64* __restrict__ X, u64 stride, u64 n, u64 W, u64 tiles,
-           u64 L, CT* __restrict__ C, u64 ldc, u32* err, long long budget)
+k_prod_tc2(const __grid_constant__ CUtensorMap map, const u64* __restrict__ X, u64 stride, u64 n, u64 W,
+           const u64* Wdev, u64 tiles, u64 L, CT* __restrict__ C, u64 ldc, u32* err, long long budget)
 {
+    if (Wdev) W = min(W, *Wdev);  // (the words up to the bound are zeros)
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) u64 full_bar[kBufs], ready_bar[kBufs], empty_bar[kBufs], ldf_bar[kSlots],
         lde_bar[kSlots], accf_bar, acce_bar, done_bar;
@@ -779,7 +780,7 @@ cudaError_t run(ProductArgs& a, const CUtensorMap& map, cudaStream_t st)
         if (dev < kMaxDevices) resident_by_dev[dev].store(nc, std::memory_order_relaxed);
     }
     const u64 clusters = std::min<u64>((u64)std::min(resident, a.sms / 2), total);
-    k_prod_tc2<CT, TMA><<<(unsigned)(2 * clusters), kThreads, kSmemBytes, st>>>(map, a.X, a.stride, a.n, a.W, tiles, L,
+    k_prod_tc2<CT, TMA><<<(unsigned)(2 * clusters), kThreads, kSmemBytes, st>>>(map, a.X, a.stride, a.n, a.W, a.Wdev, tiles, L,
                                                                           (CT*)a.C, a.ldc, a.err, wait_budget(a.timeout_ms));
     a.launches += 1;
     return cudaGetLastError();

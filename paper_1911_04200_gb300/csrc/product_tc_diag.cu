@@ -75,6 +75,7 @@ struct DiagParams {
     CUtensorMap map[kMaxDiag];
     void* C[kMaxDiag];
     u64 n[kMaxDiag], W[kMaxDiag], ldc[kMaxDiag];
+    const u64* Wdev[kMaxDiag];  // optional: the words of the job, W their bound (zeros between)
     u32 njobs;
 };
 
@@ -169,7 +170,8 @@ k_prod_diag(const __grid_constant__ DiagParams P, u32* err, long long budget)
     if (tid == 0) {
         u64 U = 0;
         for (u32 j = 0; j < njobs; ++j) {
-            ji[j] = tcs::job_info(P.n[j], P.W[j], U, kRows, kStageWords);
+            const u64 W = P.Wdev[j] ? min(P.W[j], *P.Wdev[j]) : P.W[j];
+            ji[j] = tcs::job_info(P.n[j], W, U, kRows, kStageWords);
             U += ji[j].tiles * ji[j].nst;
         }
         s_T = tcs::cta_stages(U, gridDim.x, blockIdx.x);
@@ -448,10 +450,11 @@ cudaError_t product_tc_diag(const TcJobDesc* jobs, int njobs, int count_bits, in
         P.njobs = (u32)std::min(kMaxDiag, njobs - j0);
         for (u32 j = 0; j < P.njobs; ++j) {
             const TcJobDesc& d = jobs[j0 + j];
-            if (d.Wdev || d.n > (u64)kRows) return cudaErrorInvalidValue;
+            if (d.n > (u64)kRows) return cudaErrorInvalidValue;
             P.C[j] = d.C;
             P.n[j] = d.n;
             P.W[j] = d.W;
+            P.Wdev[j] = d.Wdev;
             P.ldc[j] = d.ldc;
             if (d.n && d.W && !packed_map(&P.map[j], d.X, d.n, d.W, d.stride, kStageWords, CU_TENSOR_MAP_SWIZZLE_NONE))
                 return cudaSuccess;  // not taken (before the first launch: all jobs share one matrix's alignment)
