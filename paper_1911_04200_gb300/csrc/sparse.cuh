@@ -84,9 +84,10 @@ double pair_product_ms(u64 n, double rows)
     const double tt = (double)((n + 255) / 256);
     return tt * (tt + 1.0) / 2.0 * 65536.0 * rows / kPairMacsPerMs;
 }
-// What the order of the samples takes, and with the sketch before it.
+// What the order of the samples takes, and with the sketch before it and the
+// classification that weighs it behind it (0.25 and 0.15).
 double order_ms(u64 n) { return 0.05 + 0.7e-3 * (double)n; }
-double sketch_ms(u64 n) { return 0.2 + order_ms(n); }
+double sketch_ms(u64 n) { return 0.4 + order_ms(n); }
 // Ranked ingest: at most this many values (a 32-bit row number is kept for
 // each: 4 GiB).
 constexpr u64 kRankMaxValues = 1ull << 30;
