@@ -361,6 +361,9 @@ static int batched_body(jsim_ctx* ctx, const jsim_sets* cols, uint64_t k, void* 
                     StageTimer t(ctx, &ctx->stats.ms_product);
                     CK(cudaGraphLaunch(w.exec, ctx->stream));
                 }
+                // nothing is written when a bounded device wait ran out, as on the captured call
+                const int rcw = check_device_waits(ctx, ctx->d_err);
+                if (rcw) return rcw;
                 if (sizes)
                     for (u64 c = 0; c < k; ++c)
                         if (sizes[c] && w.cols[c].n)
