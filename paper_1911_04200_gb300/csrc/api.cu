@@ -256,6 +256,9 @@ int all_pairs_impl(jsim_ctx* ctx, const jsim_sets* sets, void* C, uint64_t* size
         if (rc) return rc;
         st.minid = fminid;
         st.maxid = fmaxid;
+        unsigned long long probes[kProbes];
+        for (int i = 0; i < kProbes; ++i) probes[i] = sets->ids[probe_place(i, st.N)];
+        set_probes(st, probes);
         feed.reset(new InputFeed());
         rc = feed->start(ctx, st, hv, feed_mt, fminid, fmaxid);
         if (rc) return rc;
@@ -295,7 +298,7 @@ int all_pairs_impl(jsim_ctx* ctx, const jsim_sets* sets, void* C, uint64_t* size
     u64 mt = 0, b_beg = 0, b_end = 0;
     const u64 v0 = st.N ? st.minid : 0, v1 = st.N ? st.maxid : 0;
     // (a part keeps the width jsim_partition_batches cuts the batches by)
-    u64 width = parts == 1 && !counts_only ? dense_batch_rows(ctx, n, st.N, v0, v1) : ctx->opt.batch_rows;
+    u64 width = parts == 1 && !counts_only ? dense_batch_rows(ctx, n, st.N, v0, v1, &st.probes) : ctx->opt.batch_rows;
     partition_rows(v0, v1, width, part, parts, b_beg, b_end, mt);
     int variant = ctx->opt.variant;
     if (st.N && b_beg < b_end) {

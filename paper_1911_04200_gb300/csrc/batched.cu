@@ -484,7 +484,7 @@ replan:
                 return JSIM_ERR_UNSUPPORTED;  // value span too wide for one batched plan
             if (widest > x.mt && !x.empty && !ctx->opt.batch_rows)
                 x.mt = std::max(x.mt, std::min(widest, dense_batch_rows(ctx, x.n, x.N, x.minid, x.maxid, nullptr,
-                                                                        kWaveBatchMs, kLanes)));
+                                                                        nullptr, kWaveBatchMs, kLanes)));
             x.lo0 = x.empty ? 0 : x.minid / x.mt * x.mt;
             x.rounds = x.empty ? 0 : x.maxid / x.mt - x.minid / x.mt + 1;
             // sum_l ceil(R_l / 64) <= N / 64 + rounds

@@ -102,13 +102,23 @@ cudaError_t launch_win_pack(const u64* ids, u64 N, const WinGeom& g, const u64* 
 // perm (optional): entry i of the plan describes sample perm[i].  ends
 // (optional): sample i's values are searched in [offsets[i], ends[i]) instead
 // of [offsets[i], offsets[i + 1]) (a slice of every sample, e.g. the part of
-// the input already copied to the device).
+// the input already copied to the device).  probes (optional, here and below;
+// N > 0 values in all): kProbes values, one of every kProbes-th part of ids.
+constexpr int kProbes = 128;
+// (at no fixed place of its part: samples that are a whole number of parts
+// long would be probed at the same few of their quantiles)
+__host__ __device__ inline u64 probe_place(u64 i, u64 N)
+{
+    return i * N / kProbes + (u64)(((unsigned __int128)(N / kProbes) * (u32)((u32)i * 2654435769u)) >> 32);
+}
 cudaError_t launch_plan(const u64* offsets, const u64* ids, u64 n, u64 lo, u64 hi, bool full,
-                        Plan plan, cudaStream_t st, const u32* perm = nullptr, const u64* ends = nullptr);
+                        Plan plan, cudaStream_t st, const u32* perm = nullptr, const u64* ends = nullptr,
+                        u64* probes = nullptr, u64 N = 0);
 // out[0] = smallest first value, out[1] = largest last value of the
 // non-empty samples (the minimum and maximum when they are sorted); out must
 // hold {~0, 0} before.
-cudaError_t launch_first_last(const u64* offsets, const u64* ids, u64 n, u64* out, cudaStream_t st);
+cudaError_t launch_first_last(const u64* offsets, const u64* ids, u64 n, u64* out, cudaStream_t st,
+                              u64* probes = nullptr, u64 N = 0);
 // err_stride 0: one error word for all samples; 1: err[i] per sample
 cudaError_t launch_validate(const u64* offsets, const u64* ids, u64 n, Plan plan, u64 max_chunks,
                             int id_bits, u64* sizes, u32* err, u64* maxid, u64* minid, int sms,

@@ -5,6 +5,7 @@
 #include <cstring>
 #include <vector>
 #include <algorithm>
+#include <cmath>
 #include "common.cuh"
 
 using namespace jsim;
@@ -266,7 +267,8 @@ struct Staged {
     DevBuf off_buf, ids_buf;
     DevBuf sizes;     // [n] distinct counts
     DevBuf plan_buf;  // beg, len, cofs, totals
-    DevBuf flags;     // validation: error word, max value, min value
+    DevBuf flags;     // validation: error word, max value, min value (then the probes)
+    std::vector<u64> probes;  // some of the values, sorted (none: not taken)
     Plan plan{};
     u64 n = 0, N = 0, maxid = 0, minid = 0, max_size = 0, max_chunks = 0;
 };
@@ -312,7 +314,7 @@ int stage_input(jsim_ctx* ctx, const jsim_sets* s, Staged& st, const std::vector
     }
     ALLOC(st.sizes, std::max<u64>(st.n, 1) * sizeof(u64));
     ALLOC(st.plan_buf, plan_words(st.n) * sizeof(u64));
-    ALLOC(st.flags, 3 * sizeof(u64));  // err (u32 in a u64), max value, min value
+    ALLOC(st.flags, (3 + kProbes) * sizeof(u64));  // err (u32 in a u64), max value, min value, probes
     st.plan = carve_plan(st.plan_buf, st.n);
     st.max_chunks = st.N / kChunk + st.n + 1;
     return JSIM_OK;
@@ -333,29 +335,41 @@ int validate_init(jsim_ctx* ctx, Staged& st, cudaStream_t vs)
 // ends null: to the sample's end), adding to the sizes and flags; slices of
 // several calls that tile every sample validate it as one call would (a
 // value is compared with the one before it in its sample, wherever that is).
-int validate_slices(jsim_ctx* ctx, Staged& st, cudaStream_t vs, const u64* begs, const u64* ends)
+int validate_slices(jsim_ctx* ctx, Staged& st, cudaStream_t vs, const u64* begs, const u64* ends,
+                    bool probe = false)
 {
-    CK(launch_plan(begs, st.d_ids, st.n, 0, 0, true, st.plan, vs, nullptr, ends));
+    CK(launch_plan(begs, st.d_ids, st.n, 0, 0, true, st.plan, vs, nullptr, ends,
+                   probe ? st.flags.as<u64>() + 3 : nullptr, st.N));
     CK(launch_validate(st.d_off, st.d_ids, st.n, st.plan, st.max_chunks, ctx->opt.id_bits, st.sizes.as<u64>(),
                        st.flags.as<u32>(), st.flags.as<u64>() + 1, st.flags.as<u64>() + 2, ctx->sms, vs));
     ctx->stats.launches += 2;
     return JSIM_OK;
 }
 
-int validate_staged(jsim_ctx* ctx, Staged& st, cudaStream_t vs)
+int validate_staged(jsim_ctx* ctx, Staged& st, cudaStream_t vs, bool probe = false)
 {
     int rc = validate_init(ctx, st, vs);
     if (rc) return rc;
-    return validate_slices(ctx, st, vs, st.d_off, nullptr);
+    return validate_slices(ctx, st, vs, st.d_off, nullptr, probe);
+}
+
+// The probes of a range (minid, maxid set) that takes more than one batch.
+void set_probes(Staged& st, const unsigned long long* v)
+{
+    if (st.maxid - st.minid < (1ull << 28)) return;
+    st.probes.assign(v, v + kProbes);
+    std::sort(st.probes.begin(), st.probes.end());
 }
 
 // The validation's verdict (after the context's stream has waited for it):
 // JSIM_ERR_UNSORTED, JSIM_ERR_ID_RANGE, JSIM_ERR_OVERFLOW (a size that 32-bit
-// counts cannot hold), or st.minid, st.maxid and st.max_size.
-int check_staged(jsim_ctx* ctx, Staged& st)
+// counts cannot hold), or st.minid, st.maxid and st.max_size (with probe, and
+// st.probes).
+int check_staged(jsim_ctx* ctx, Staged& st, bool probe = false)
 {
     std::vector<u64> hs(st.n);
-    CK(cudaMemcpyAsync(ctx->h_scalars, st.flags.p, 3 * sizeof(u64), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaMemcpyAsync(ctx->h_scalars, st.flags.p, (3 + (probe ? kProbes : 0)) * sizeof(u64), cudaMemcpyDeviceToHost,
+                       ctx->stream));
     CK(cudaMemcpyAsync(hs.data(), st.sizes.p, st.n * sizeof(u64), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     u32 f = (u32)ctx->h_scalars[0];
@@ -363,6 +377,7 @@ int check_staged(jsim_ctx* ctx, Staged& st)
     if (f & kFlagIdRange) return JSIM_ERR_ID_RANGE;
     st.maxid = ctx->h_scalars[1];
     st.minid = ctx->h_scalars[2];
+    if (probe) set_probes(st, ctx->h_scalars + 3);
     st.max_size = 0;
     for (u64 v : hs) st.max_size = std::max(st.max_size, v);
     if (ctx->opt.count_bits == 32 && st.max_size > 0xffffffffull) return JSIM_ERR_OVERFLOW;
@@ -430,18 +445,21 @@ struct SideValidation {
 
 // The smallest first and largest last value of the staged samples (their
 // minimum and maximum when sorted) into st.minid and st.maxid; none: {~0, 0}.
+// Also st.probes.
 int first_last_values(jsim_ctx* ctx, Staged& st)
 {
     DevBuf fl;
-    ALLOC(fl, 2 * sizeof(u64));
+    ALLOC(fl, (2 + kProbes) * sizeof(u64));
     CK(cudaMemsetAsync(fl.p, 0xff, sizeof(u64), ctx->stream));
     CK(cudaMemsetAsync(fl.as<u64>() + 1, 0, sizeof(u64), ctx->stream));
-    CK(launch_first_last(st.d_off, st.d_ids, st.n, fl.as<u64>(), ctx->stream));
+    CK(launch_first_last(st.d_off, st.d_ids, st.n, fl.as<u64>(), ctx->stream, st.N ? fl.as<u64>() + 2 : nullptr, st.N));
     ctx->stats.launches += 1;
-    CK(cudaMemcpyAsync(ctx->h_scalars, fl.p, 2 * sizeof(u64), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaMemcpyAsync(ctx->h_scalars, fl.p, (2 + (st.N ? kProbes : 0)) * sizeof(u64), cudaMemcpyDeviceToHost,
+                       ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     st.minid = ctx->h_scalars[0];
     st.maxid = ctx->h_scalars[1];
+    if (st.N) set_probes(st, ctx->h_scalars + 2);
     return JSIM_OK;
 }
 
@@ -453,10 +471,10 @@ int stage_and_validate(jsim_ctx* ctx, const jsim_sets* s, Staged& st, const std:
     if (rc) return rc;
     {
         StageTimer t(ctx, &ctx->stats.ms_validate);
-        rc = validate_staged(ctx, st, ctx->stream);
+        rc = validate_staged(ctx, st, ctx->stream, st.N > 0);
         if (rc) return rc;
     }
-    return check_staged(ctx, st);
+    return check_staged(ctx, st, st.N > 0);
 }
 
 // Largest power-of-two batch up to 2^28 rows (its 32 MiB filter bitmap and
@@ -486,20 +504,54 @@ u64 auto_batch_rows(u64 domain)
 // So few values take wide batches and many take 2^28 rows.  A batch is wider
 // than 2^28 only where its packed matrix is small (bounded by its values) and
 // the device has room for its bitmaps.
+//
+// That is for values spread over the whole range.  Stretches that hold none
+// cost nothing (the loop goes on at the next value), so where the values leave
+// half of the range's narrow batches empty or more, a batch is also charged
+// for what it clears and scans (kDenseRowMs).  16 samples of 500 values of
+// [0, 2^64) (1000 batches of either width): 286 ms in 2^32-row batches, 66 in
+// 2^28; three clusters 2^33 apart or more, 8e5 values: 1.19 and 0.47; spread
+// over [0, 2^40), 3.2e5 values: 74 and 307.
 constexpr double kDenseBatchMs = 0.17;
 constexpr double kDenseValueMs[2][5] = {{2.8e-8, 3.4e-8, 5.0e-8, 7.0e-8, 8.2e-8},   // one filter
                                         {2.8e-8, 3.9e-8, 6.1e-8, 8.2e-8, 9.8e-8}};  // two-or-more
-// (batch_ms: kDenseBatchMs, or what else a batch costs the caller; copies: how
-// many sets of bitmaps it keeps)
-u64 dense_batch_rows(const jsim_ctx* ctx, u64 n, u64 N, u64 minid, u64 maxid, double* ms = nullptr,
-                     double batch_ms = kDenseBatchMs, int copies = 1)
+constexpr double kDenseRowMs[2] = {0.24 / 4294967296.0, 0.40 / 4294967296.0};  // one filter, two-or-more
+
+// The batches of `w` rows that hold a value of [minid, maxid], as far as the
+// number of values and the sorted probes tell: D stretches among S probes of B
+// equally full ones are D = B (1 - (1 - 1/B)^S) on average, which says little
+// about B once most probes lie in stretches of their own.
+double batch_count(u64 N, u64 minid, u64 maxid, u64 w, const std::vector<u64>& probes)
+{
+    double b = std::min((double)(maxid / w - minid / w + 1), (double)N);
+    const double S = (double)probes.size();
+    if (probes.empty()) return b;
+    double D = 1;
+    for (size_t i = 1; i < probes.size(); ++i) D += probes[i] / w != probes[i - 1] / w;
+    if (D > 0.75 * S) return b;
+    double est = D;
+    while (est < b && est * (1.0 - std::pow(1.0 - 1.0 / est, S)) < D - 0.5) est *= 1.05;
+    est += (minid / w != probes.front() / w) + (maxid / w != probes.back() / w);
+    return std::min(b, est);
+}
+
+// (probes: of the values, where the caller skips empty stretches; batch_ms:
+// kDenseBatchMs, or what else a batch costs the caller; copies: how many sets
+// of bitmaps it keeps)
+u64 dense_batch_rows(const jsim_ctx* ctx, u64 n, u64 N, u64 minid, u64 maxid, const std::vector<u64>* probes,
+                     double* ms = nullptr, double batch_ms = kDenseBatchMs, int copies = 1)
 {
     const u64 span = maxid - minid;
-    const double* value_ms = kDenseValueMs[ctx->opt.filter_min == 2];
-    auto cost = [&](u64 w, int k) {
-        return (double)(maxid / w - minid / w + 1) * batch_ms + (double)N * value_ms[k];
-    };
+    const bool twice = ctx->opt.filter_min == 2;
+    const double* value_ms = kDenseValueMs[twice];
     u64 best = ctx->opt.batch_rows ? ctx->opt.batch_rows : auto_batch_rows(span + 1 ? span + 1 : ~0ull);
+    auto all = [&](u64 w) { return (double)(maxid / w - minid / w + 1); };
+    const bool holes = probes && 2.0 * batch_count(N, minid, maxid, best, *probes) < all(best);
+    auto cost = [&](u64 w, int k) {
+        return (holes ? batch_count(N, minid, maxid, w, *probes) * (batch_ms + (double)w * kDenseRowMs[twice])
+                      : all(w) * batch_ms) +
+               (double)N * value_ms[k];
+    };
     double best_ms = cost(best, 0);
     size_t free_b = 0, total_b = 0;
     for (int k = 1; k < 5 && !ctx->opt.batch_rows; ++k) {
@@ -507,9 +559,17 @@ u64 dense_batch_rows(const jsim_ctx* ctx, u64 n, u64 N, u64 minid, u64 maxid, do
         if (w / 2 > span) break;
         const double t = cost(w, k);
         if (t >= best_ms) continue;
-        const double held = std::min(1.0, (double)w / ((double)span + 1.0)) * (double)N;
+        double held = std::min(1.0, (double)w / ((double)span + 1.0)) * (double)N;
+        if (holes && !probes->empty()) {  // the fullest batch the probes show
+            size_t most = 0, run = 0;
+            for (size_t i = 0; i < probes->size(); ++i) {
+                run = i && (*probes)[i] / w == (*probes)[i - 1] / w ? run + 1 : 1;
+                most = std::max(most, run);
+            }
+            held = std::max(held, (double)N * (double)most / (double)probes->size());
+        }
         const double x_bytes = (double)round_up(std::max<u64>(n, 1), kRowPad) * held / 8.0;
-        const double bytes = x_bytes + copies * (double)w / 8.0 * (ctx->opt.filter_min == 2 ? 2.5 : 1.5);
+        const double bytes = x_bytes + copies * (double)w / 8.0 * (twice ? 2.5 : 1.5);
         if (!total_b && cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) { cudaGetLastError(); break; }
         if (x_bytes > (double)(4ull << 30) || bytes > (double)free_b / 4.0) continue;
         best = w;

@@ -76,6 +76,13 @@ __device__ __forceinline__ void plan_search(const u64* __restrict__ offsets, con
     }
 }
 
+// kProbes values (null: none).
+__device__ __forceinline__ void take_probes(const u64* __restrict__ ids, u64 N, u64* probes)
+{
+    static_assert(kProbes <= kPlanThreads, "a probe a thread");
+    if (probes && threadIdx.x < kProbes) probes[threadIdx.x] = ids[probe_place(threadIdx.x, N)];
+}
+
 // One CTA: per-sample [beg, beg+len) of values in [lo, hi) and chunk prefix.
 // With perm, entry i of the plan is sample perm[i] (the ingest kernels then
 // walk the samples in that order).  With ends, sample i is searched in
@@ -83,8 +90,9 @@ __device__ __forceinline__ void plan_search(const u64* __restrict__ offsets, con
 // samples of 50,000 values 24.6 us by bisection, 9 us here.
 __global__ void __launch_bounds__(kPlanThreads)
 k_plan(const u64* __restrict__ offsets, const u64* __restrict__ ids, u64 n, u64 lo, u64 hi,
-       int full, Plan plan, const u32* __restrict__ perm, const u64* __restrict__ ends)
+       int full, Plan plan, const u32* __restrict__ perm, const u64* __restrict__ ends, u64* probes, u64 N)
 {
+    take_probes(ids, N, probes);
     __shared__ u64 sm[kPlanThreads / 32];
     __shared__ u64 s_next;
     __shared__ int s_has_next;
@@ -599,8 +607,9 @@ k_pack_classes(const u64* __restrict__ ids, const u32* __restrict__ ranks, u64 n
 // samples (for sorted samples: the collection's minimum and maximum); out
 // must hold {~0, 0} before.  One CTA.
 __global__ void __launch_bounds__(kPlanThreads)
-k_first_last(const u64* __restrict__ offsets, const u64* __restrict__ ids, u64 n, u64* out)
+k_first_last(const u64* __restrict__ offsets, const u64* __restrict__ ids, u64 n, u64* out, u64* probes, u64 N)
 {
+    take_probes(ids, N, probes);
     __shared__ unsigned long long s_min, s_max;
     if (threadIdx.x == 0) { s_min = ~0ull; s_max = 0ull; }
     __syncthreads();
@@ -631,9 +640,9 @@ inline unsigned grid_for_chunks(u64 max_chunks, int sms)
 }  // namespace
 
 cudaError_t launch_plan(const u64* offsets, const u64* ids, u64 n, u64 lo, u64 hi, bool full,
-                        Plan plan, cudaStream_t st, const u32* perm, const u64* ends)
+                        Plan plan, cudaStream_t st, const u32* perm, const u64* ends, u64* probes, u64 N)
 {
-    k_plan<<<1, kPlanThreads, 0, st>>>(offsets, ids, n, lo, hi, full ? 1 : 0, plan, perm, ends);
+    k_plan<<<1, kPlanThreads, 0, st>>>(offsets, ids, n, lo, hi, full ? 1 : 0, plan, perm, ends, probes, N);
     return cudaGetLastError();
 }
 
@@ -713,9 +722,9 @@ cudaError_t launch_pack_classes(const u64* ids, const u32* ranks, u64 n, Plan pl
     return cudaGetLastError();
 }
 
-cudaError_t launch_first_last(const u64* offsets, const u64* ids, u64 n, u64* out, cudaStream_t st)
+cudaError_t launch_first_last(const u64* offsets, const u64* ids, u64 n, u64* out, cudaStream_t st, u64* probes, u64 N)
 {
-    k_first_last<<<1, kPlanThreads, 0, st>>>(offsets, ids, n, out);
+    k_first_last<<<1, kPlanThreads, 0, st>>>(offsets, ids, n, out, probes, N);
     return cudaGetLastError();
 }
 

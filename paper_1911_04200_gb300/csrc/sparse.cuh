@@ -379,7 +379,7 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
     // where the model says so, and in place of the per-value ingest wherever
     // the batches' width is free.
     double dense_ingest = 0;
-    const u64 dense_mt = st.N ? dense_batch_rows(ctx, n, st.N, st.minid, st.maxid, &dense_ingest) : 0;
+    const u64 dense_mt = st.N ? dense_batch_rows(ctx, n, st.N, st.minid, st.maxid, &st.probes, &dense_ingest) : 0;
     const double windowed_ms = ((double)span + 1.0) / 4294967296.0 * (double)T * kWinTileMs[twice] +
                                (double)st.N * kWinValueMs[twice];
     bool windowed = false, ranked = st.N && st.N <= kRankMaxValues && !ctx->opt.batch_rows;
@@ -390,13 +390,12 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
         if (ranked && windowed && (per_window >= kWinSureValues || windowed_ms <= dense_ingest)) ranked = false;
         if (ranked) windowed = false;
         mt = feed ? feed->mt : ranked ? std::max(kMinClassRows, dense_mt) : sparse_batch_rows(ctx, n, span, windowed);
-        sparse_ingest = ranked     ? (feed ? (double)(st.maxid / mt - st.minid / mt + 1) * kDenseBatchMs +
+        const double batches = st.N && mt ? batch_count(st.N, st.minid, st.maxid, mt, st.probes) : 0.0;
+        sparse_ingest = ranked     ? (feed ? batches * kDenseBatchMs +
                                                 (double)st.N * kDenseValueMs[twice][0]
                                           : dense_ingest)
                         : windowed ? windowed_ms
-                        : mt       ? (double)(st.maxid / mt - st.minid / mt + 1) * kPerBatchMs[twice] +
-                                   (double)st.N * kPerValueMs
-                                   : 0.0;
+                                   : batches * kPerBatchMs[twice] + (double)st.N * kPerValueMs;
     };
     choose_ingest();
     if (!mt) return JSIM_ERR_UNSUPPORTED;
