@@ -347,9 +347,10 @@ u64 feed_batch_rows(const jsim_ctx* ctx, u64 n, u64 N, u64 span)
 // is validated when the last piece is in); with sv, the values are there and
 // their validation runs beside the sketch and the batches.  Either way
 // st.minid and st.maxid are every sample's first and last value until the
-// verdict is read, before any output is written.
-int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double* J, int out_mem,
-                     bool may_decline, bool& declined, InputFeed* feed = nullptr, SideValidation* sv = nullptr)
+// verdict is read, before any output is written.  ranked: whether the ranked
+// ingest may be taken, and on return whether it was.
+int all_pairs_sparse_with(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double* J, int out_mem,
+                          bool may_decline, bool& declined, InputFeed* feed, SideValidation* sv, bool& ranked)
 {
     declined = false;
     const u64 n = st.n;
@@ -382,23 +383,20 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
     const u64 dense_mt = st.N ? dense_batch_rows(ctx, n, st.N, st.minid, st.maxid, &st.probes, &dense_ingest) : 0;
     const double windowed_ms = ((double)span + 1.0) / 4294967296.0 * (double)T * kWinTileMs[twice] +
                                (double)st.N * kWinValueMs[twice];
-    bool windowed = false, ranked = st.N && st.N <= kRankMaxValues && !ctx->opt.batch_rows;
-    u64 mt = 0;
-    double sparse_ingest = 0;
-    auto choose_ingest = [&]() {
-        windowed = per_window >= kWinMinValues && !feed;
-        if (ranked && windowed && (per_window >= kWinSureValues || windowed_ms <= dense_ingest)) ranked = false;
-        if (ranked) windowed = false;
-        mt = feed ? feed->mt : ranked ? std::max(kMinClassRows, dense_mt) : sparse_batch_rows(ctx, n, span, windowed);
-        const double batches = st.N && mt ? batch_count(st.N, st.minid, st.maxid, mt, st.probes) : 0.0;
-        sparse_ingest = ranked     ? (feed ? batches * kDenseBatchMs +
-                                                (double)st.N * kDenseValueMs[twice][0]
-                                          : dense_ingest)
-                        : windowed ? windowed_ms
-                                   : batches * kPerBatchMs[twice] + (double)st.N * kPerValueMs;
-    };
-    choose_ingest();
+    bool windowed = per_window >= kWinMinValues && !feed;
+    ranked = ranked && st.N && st.N <= kRankMaxValues && !ctx->opt.batch_rows;
+    if (ranked && windowed && (per_window >= kWinSureValues || windowed_ms <= dense_ingest)) ranked = false;
+    if (ranked) windowed = false;
+    u64 mt = ranked ? std::max(kMinClassRows, dense_mt) : sparse_batch_rows(ctx, n, span, windowed);
+    // (a feed's pieces are whole batches of feed->mt; both widths are powers of
+    // two, or the caller's one)
+    if (feed) mt = ranked ? feed->mt : std::min(mt, feed->mt);
     if (!mt) return JSIM_ERR_UNSUPPORTED;
+    const double batches = st.N ? batch_count(st.N, st.minid, st.maxid, mt, st.probes) : 0.0;
+    const double sparse_ingest = ranked ? (feed ? batches * kDenseBatchMs + (double)st.N * kDenseValueMs[twice][0]
+                                                : dense_ingest)
+                                 : windowed ? windowed_ms
+                                            : batches * kPerBatchMs[twice] + (double)st.N * kPerValueMs;
     ctx->stats.batch_rows = mt;
     // The call's time dense with `rows` nonzero rows, and block-sparse with
     // `prod` ms of products.  A value is at most one row (with the two-or-more
@@ -415,14 +413,12 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
     DevBuf rk_bits, rk_seen, rk_dir, rk_bsum, rk_boff, ranks;
     if (ranked) {
         const u64 nw = mt / 64, nb = (nw + kScanBlockWords - 1) / kScanBlockWords;
-        ranked = rk_bits.ensure(ctx, nw * 8) && (!twice || rk_seen.ensure(ctx, nw * 8)) && rk_dir.ensure(ctx, nw * 4) &&
-                 rk_bsum.ensure(ctx, nb * 8) && rk_boff.ensure(ctx, nb * 8) && ranks.ensure(ctx, st.N * 4);
-        if (!ranked) {  // no room for it: the other ingests hold less
-            for (DevBuf* b : {&rk_bits, &rk_seen, &rk_dir, &rk_bsum, &rk_boff, &ranks}) b->release();
-            choose_ingest();
-            if (!mt) return JSIM_ERR_UNSUPPORTED;
-            ctx->stats.batch_rows = mt;
-        }
+        ALLOC(rk_bits, nw * 8);
+        if (twice) ALLOC(rk_seen, nw * 8);
+        ALLOC(rk_dir, nw * 4);
+        ALLOC(rk_bsum, nb * 8);
+        ALLOC(rk_boff, nb * 8);
+        ALLOC(ranks, st.N * 4);
     }
 
     // search bounds of a batch at lo: with a feed, the slices of lo's piece
@@ -1002,6 +998,24 @@ int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double
     }
     CK(cudaStreamSynchronize(cs));
     return JSIM_OK;
+}
+
+// The path with the ingest the call's values ask for.  The ranked ingest holds
+// more than the others (a row number a value, the bitmap and directory of a
+// wide batch, classes as wide as the batch's rows): where any request of it is
+// refused, the call starts over without it.  Nothing has been written then.
+int all_pairs_sparse(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, double* J, int out_mem,
+                     bool may_decline, bool& declined, InputFeed* feed = nullptr, SideValidation* sv = nullptr)
+{
+    const jsim_stats before = ctx->stats;
+    bool ranked = true;
+    int rc = all_pairs_sparse_with(ctx, st, C, sizes, J, out_mem, may_decline, declined, feed, sv, ranked);
+    if (rc == JSIM_ERR_OOM && ranked) {
+        ctx->stats = before;
+        ranked = false;
+        rc = all_pairs_sparse_with(ctx, st, C, sizes, J, out_mem, may_decline, declined, feed, sv, ranked);
+    }
+    return rc;
 }
 
 }  // namespace
