@@ -502,7 +502,7 @@ replan:
         w.batches = batches;
         return JSIM_OK;
     };
-    auto alloc_lanes = [&]() -> int {
+    auto alloc_wave = [&]() -> int {
         const u64 nwords = std::max<u64>(w.max_mt / 64, 1);
         const u64 nb = (nwords + kScanBlockWords - 1) / kScanBlockWords;
         for (int l = 0; l < kLanes; ++l) {
@@ -512,6 +512,14 @@ replan:
             ALLOC(w.bsum[l], std::max<u64>(nb, 1) * 8);
             ALLOC(w.boff[l], std::max<u64>(nb, 1) * 8);
             ALLOC(w.R[l], 8);
+        }
+        ALLOC(w.xpool, std::max<size_t>(x_tot, 1) * 8);
+        ALLOC(w.cpool, std::max<size_t>(c_tot, 8));
+        ALLOC(w.scal, 2 * sizeof(u64) * k);
+        ALLOC(w.jobtab, sizeof(TcJobDesc) * std::max<u64>(k, 1));
+        if (!dev_out) {
+            if (C) ALLOC(w.cstage, std::max<size_t>(cs_tot, 8));
+            if (J) ALLOC(w.jstage, std::max<size_t>(js_tot, 8));
         }
         return JSIM_OK;
     };
@@ -526,28 +534,22 @@ replan:
             rc = plan_wave(widest);
             if (rc) return rc;
         }
-        rc = alloc_lanes();
-        if (rc == JSIM_ERR_OOM && w.max_mt > narrow && !ctx->opt.batch_rows) {  // no room for the wide batches
+        rc = alloc_wave();
+        if (rc == JSIM_ERR_OOM && w.max_mt > narrow && !ctx->opt.batch_rows) {
+            // no room for the wide batches and what lies behind them
             for (int l = 0; l < kLanes; ++l)
                 for (DevBuf* d : {&w.bitmap[l], &w.seen[l], &w.dir[l], &w.bsum[l], &w.boff[l]}) d->release();
+            for (DevBuf* d : {&w.xpool, &w.cpool, &w.scal, &w.jobtab, &w.cstage, &w.jstage}) d->release();
             rc = plan_wave(narrow);
-            if (!rc) rc = alloc_lanes();
+            if (!rc) rc = alloc_wave();
         }
         if (rc) return rc;
         ctx->stats.batches += w.batches;
-        ALLOC(w.xpool, std::max<size_t>(x_tot, 1) * 8);
-        ALLOC(w.cpool, std::max<size_t>(c_tot, 8));
-        ALLOC(w.scal, 2 * sizeof(u64) * k);
-        ALLOC(w.jobtab, sizeof(TcJobDesc) * std::max<u64>(k, 1));
         std::vector<TcJobDesc> jobs = wave_jobs(w);
         if (!jobs.empty())
             CK(cudaMemcpyAsync(w.jobtab.p, jobs.data(), sizeof(TcJobDesc) * jobs.size(), cudaMemcpyHostToDevice,
                                ctx->stream));
         CK(cudaStreamSynchronize(ctx->stream));
-        if (!dev_out) {
-            if (C) ALLOC(w.cstage, std::max<size_t>(cs_tot, 8));
-            if (J) ALLOC(w.jstage, std::max<size_t>(js_tot, 8));
-        }
     }
 
     // ---- variant: the caller's, or the tuned one for this shape ----

@@ -163,3 +163,26 @@ def test_ranked_ingest_of_fed_input_gives_way(gpu):
     assert not a.live
     assert (C == C2).all() and (s == s2).all() and (J.view(np.uint64) == J2.view(np.uint64)).all()
     np.testing.assert_array_equal(s, oracle.sizes_of(off, ids))
+
+
+@pytest.mark.timeout(300)
+@pytest.mark.parametrize("filter_min", [1, 2])
+def test_wide_batches_of_a_batched_call_give_way(gpu, filter_min):
+    """The wide lanes are granted and the last buffer behind them is refused."""
+    cols = [spread_sets(n, 30_000, 32, seed=n) for n in (250, 249, 248, 247, 246, 245, 244, 40)]
+    kw = dict(variant="popc", filter_min=filter_min)
+    a = Capped()
+    with jsim.Context(allocator=a, **kw) as ctx:
+        refs = ctx.all_pairs_batched(cols)
+        rounds = ctx.stats()["batches"]
+    assert rounds < 8 * len(cols)  # (8 batches of 2^29 rows each)
+    Co, so, Jo = oracle.all_pairs(*cols[-1])
+    assert_same(refs[-1], (Co, so, Jo))
+    b = Capped(total=a.peak - 1)
+    with jsim.Context(allocator=b, **kw) as ctx:
+        outs = ctx.all_pairs_batched(cols)
+        assert b.refused and ctx.stats()["batches"] == 8 * len(cols)
+    for res, ref in zip(outs, refs):
+        for x, y in zip(res, ref):
+            np.testing.assert_array_equal(x.view(np.uint8), y.view(np.uint8))
+    assert not b.live
