@@ -563,6 +563,10 @@ replan:
     u64 shape = 0x77;
     for (auto& x : w.cols) shape = mix(shape, (x.n + 31) / 32 * 1000003 + (64 - __builtin_clzll(x.N | 1)));
     shape = mix(shape, (u64)ctx->opt.tile_n);
+    // (the 4-bit products load rows by TMA: a choice made with 16-byte aligned
+    // matrices does not hold for others)
+    const bool aligned = (uintptr_t)w.xpool.p % 16 == 0;
+    shape = mix(shape, aligned ? 1 : 0);
     if (variant == JSIM_VARIANT_AUTO) {
         for (auto& e : tun->entries)
             if (e.first == shape) {
@@ -585,7 +589,7 @@ replan:
             static_assert(kWordPad % 2 == 0, "16-byte aligned rows");
             // 4-bit operands (13 collections of 31 to 231 samples x 20,000 values,
             // whole call: 6.8 ms with byte tiles, 6.1)
-            if (!ctx->opt.tile_n && (uintptr_t)w.xpool.p % 16 == 0) cands.push_back({JSIM_VARIANT_TC2, 64, 256});
+            if (!ctx->opt.tile_n && aligned) cands.push_back({JSIM_VARIANT_TC2, 64, 256});
             if (ctx->opt.tile_n != 128) cands.push_back({JSIM_VARIANT_TC, 64, 256});
             if (ctx->opt.tile_n != 256) cands.push_back({JSIM_VARIANT_TC, 64, 128});
         }
