@@ -207,7 +207,8 @@ struct TcJobDesc {
 cudaError_t product_tc_jobs(const TcJobDesc* jobs, int njobs, void* dev_table, bool upload, int count_bits, int sms,
                             u32* err, int timeout_ms, cudaStream_t st, int* launches, int tile_n = 256);
 // Jobs of at most 128 samples each (with Wdev, W is a bound and the words past
-// *Wdev are zeros; the SM-pair product likewise), one diagonal 128 x 128 tile per job, up to 16 jobs a launch.  *taken false: a matrix's rows are not
+// *Wdev are zeros; the SM-pair product likewise), one diagonal 128 x 128 tile
+// per job, up to 16 jobs a launch.  *taken false: a matrix's rows are not
 // 16-byte aligned, and nothing was launched.
 cudaError_t product_tc_diag(const TcJobDesc* jobs, int njobs, int count_bits, int sms, u32* err, int timeout_ms,
                             cudaStream_t st, int* launches, bool* taken);

@@ -27,6 +27,7 @@
 // raises the error word, waits (bounded) for its issued MMAs and copies,
 // frees its TMEM and leaves.
 #include <algorithm>
+#include <vector>
 #include "tensor_map.cuh"
 #include "product_tc_sched.cuh"
 
@@ -445,21 +446,24 @@ cudaError_t product_tc_diag(const TcJobDesc* jobs, int njobs, int count_bits, in
                             cudaStream_t st, int* launches, bool* taken)
 {
     *taken = false;
-    for (int j0 = 0; j0 < njobs; j0 += kMaxDiag) {
-        DiagParams P{};
-        P.njobs = (u32)std::min(kMaxDiag, njobs - j0);
-        for (u32 j = 0; j < P.njobs; ++j) {
-            const TcJobDesc& d = jobs[j0 + j];
-            if (d.n > (u64)kRows) return cudaErrorInvalidValue;
-            P.C[j] = d.C;
-            P.n[j] = d.n;
-            P.W[j] = d.W;
-            P.Wdev[j] = d.Wdev;
-            P.ldc[j] = d.ldc;
-            if (d.n && d.W && !packed_map(&P.map[j], d.X, d.n, d.W, d.stride, kStageWords, CU_TENSOR_MAP_SWIZZLE_NONE))
-                return cudaSuccess;  // not taken (before the first launch: all jobs share one matrix's alignment)
-        }
-        *taken = true;
+    // every job's map before the first launch: all jobs or none
+    std::vector<DiagParams> groups((size_t)((njobs + kMaxDiag - 1) / kMaxDiag));
+    for (int q = 0; q < njobs; ++q) {
+        DiagParams& P = groups[(size_t)(q / kMaxDiag)];
+        const int j = q % kMaxDiag;
+        const TcJobDesc& d = jobs[q];
+        if (d.n > (u64)kRows) return cudaErrorInvalidValue;
+        P.njobs = (u32)j + 1;
+        P.C[j] = d.C;
+        P.n[j] = d.n;
+        P.W[j] = d.W;
+        P.Wdev[j] = d.Wdev;
+        P.ldc[j] = d.ldc;
+        if (d.n && d.W && !packed_map(&P.map[j], d.X, d.n, d.W, d.stride, kStageWords, CU_TENSOR_MAP_SWIZZLE_NONE))
+            return cudaSuccess;
+    }
+    *taken = true;
+    for (const DiagParams& P : groups) {
         const cudaError_t e = count_bits == 64 ? run<u64>(P, sms, err, timeout_ms, st)
                                                : run<u32>(P, sms, err, timeout_ms, st);
         if (e != cudaSuccess) return e;
