@@ -20,6 +20,7 @@
 // tiles, tcgen05 over the table, CUDA-core with 64-bit and 32-bit words) on the
 // first call of a collection shape and keeps the fastest for that shape.
 #include <algorithm>
+#include <memory>
 #include "ctx.cuh"
 
 namespace {
@@ -266,23 +267,37 @@ jsim_tuning* tuning_of(jsim_ctx* ctx)
     tab.push_back({ctx, new jsim_tuning()});
     return tab.back().second;
 }
-std::vector<std::pair<jsim_ctx*, Wave*>>& wave_cache()
-{
-    static std::vector<std::pair<jsim_ctx*, Wave*>> c;
-    return c;
-}
+
+// The wave kept for a replay, taken by a call (so that no request of the call
+// gives it back) and kept again when the call is done with it.
+struct KeptWave {
+    jsim_ctx* ctx;
+    std::unique_ptr<Wave> w;
+    explicit KeptWave(jsim_ctx* c) : ctx(c), w((Wave*)c->kept_wave) { c->kept_wave = nullptr; }
+    ~KeptWave() { ctx->kept_wave = w.release(); }
+};
+
+// The wave of a call that replays nothing; one that an error ends goes once the
+// side streams are through with it.
+struct FreshWave {
+    jsim_ctx* ctx;
+    std::unique_ptr<Wave> w;
+    bool done = false;
+    ~FreshWave()
+    {
+        if (done) return;
+        for (cudaStream_t s : ctx->lanes) cudaStreamSynchronize(s);
+        cudaGetLastError();
+    }
+};
 }  // namespace
 
-void jsim_batched_release(jsim_ctx* ctx)
+bool jsim_batched_release(jsim_ctx* ctx)
 {
-    auto& wc = wave_cache();
-    for (size_t i = 0; i < wc.size(); ++i) {
-        if (wc[i].first == ctx) {
-            delete wc[i].second;
-            wc.erase(wc.begin() + i);
-            --i;
-        }
-    }
+    if (!ctx->kept_wave) return false;
+    delete (Wave*)ctx->kept_wave;
+    ctx->kept_wave = nullptr;
+    return true;
 }
 
 // The batched machinery over k collections (statistics into the caller's
@@ -322,12 +337,12 @@ static int batched_body(jsim_ctx* ctx, const jsim_sets* cols, uint64_t k, void* 
     CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(u32), ctx->stream));
 
     // ---- replay a captured call on the same collections ----
-    auto& wc = wave_cache();
-    if (use_graph) {
-        for (auto& e : wc) {
-            if (e.first == ctx && e.second->signature == sig && e.second->exec) {
+    {
+        KeptWave kept(ctx);
+        if (use_graph) {
+            if (kept.w && kept.w->signature == sig && kept.w->exec) {
                 // validation still runs: the values may have changed
-                Wave& w = *e.second;
+                Wave& w = *kept.w;
                 DevBuf flags;
                 ALLOC(flags, 3 * sizeof(u64) * k);
                 CK(cudaMemsetAsync(flags.p, 0, 3 * sizeof(u64) * k, ctx->stream));
@@ -378,9 +393,8 @@ static int batched_body(jsim_ctx* ctx, const jsim_sets* cols, uint64_t k, void* 
     }
 replan:
     jsim_batched_release(ctx);
-    Wave* wp = new Wave();
-    Wave& w = *wp;
-    wc.push_back({ctx, wp});
+    FreshWave fresh{ctx, std::unique_ptr<Wave>(new Wave())};
+    Wave& w = *fresh.w;
     w.signature = sig;
     w.cols = std::move(cl);
 
@@ -658,7 +672,8 @@ replan:
     }
     CK(cudaStreamSynchronize(ctx->stream));
     int rc = finish_stats(ctx, w);
-    if (!use_graph) jsim_batched_release(ctx);  // nothing to replay: free the wave now
+    fresh.done = !rc;
+    if (use_graph && !rc) ctx->kept_wave = fresh.w.release();  // (else there is nothing to replay)
     return rc;
 }
 

@@ -16,8 +16,9 @@ struct jsim_ctx;
 // (C linkage, as the C-ABI translation unit defines it; not exported)
 extern "C" int all_pairs_impl(jsim_ctx* ctx, const jsim_sets* sets, void* C, uint64_t* sizes, double* J,
                               int out_mem, u64 part, u64 parts, bool counts_only, bool own_scope);
-// releases the batched-call state (captured graphs and buffers) of a context
-void jsim_batched_release(jsim_ctx* ctx);
+// releases what a batched call keeps for a replay (captured graph and
+// buffers); false: nothing was kept
+bool jsim_batched_release(jsim_ctx* ctx);
 // releases the streamed-call state (pinned staging, copy stream) of a context
 void jsim_streamed_release(jsim_ctx* ctx);
 struct StreamState;
@@ -44,6 +45,8 @@ struct jsim_ctx {
     size_t events_used = 0;
     struct Pending { cudaEvent_t a, b; double* acc; };
     std::vector<Pending> pending;
+    // what the last batched call keeps for a replay (not while a call uses it)
+    void* kept_wave = nullptr;
     // streamed calls: pinned staging buffers kept between calls
     StreamState* streamed = nullptr;
     // side streams for independent per-collection work (batched calls), with
@@ -95,7 +98,8 @@ struct DevBuf {
         p = nullptr;
         bytes = 0;
     }
-    // (re)allocate at least `b` bytes; contents undefined
+    // (re)allocate at least `b` bytes; contents undefined.  A refusal gives
+    // back what a batched call keeps for a replay and asks once more.
     bool ensure(jsim_ctx* c, size_t b)
     {
         if (p && bytes >= b) return true;
@@ -103,6 +107,7 @@ struct DevBuf {
         ctx = c;
         size_t bb = b ? b : 16;
         p = c->opt.alloc(bb, (void*)c->stream, c->opt.alloc_user);
+        if (!p && jsim_batched_release(c)) p = c->opt.alloc(bb, (void*)c->stream, c->opt.alloc_user);
         if (!p) return false;
         bytes = bb;
         return true;

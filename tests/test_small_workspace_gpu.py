@@ -186,3 +186,28 @@ def test_wide_batches_of_a_batched_call_give_way(gpu, filter_min):
         for x, y in zip(res, ref):
             np.testing.assert_array_equal(x.view(np.uint8), y.view(np.uint8))
     assert not b.live
+
+
+def test_a_captured_call_gives_its_buffers_back(gpu):
+    """The buffers kept for a replay make room when another call on the context
+    needs them."""
+    import torch
+    cols = [spread_sets(n, 30_000, 32, seed=n) for n in (120, 200)]
+    dev = [(torch.from_numpy(o.view(np.int64)).cuda(), torch.from_numpy(i.view(np.int64)).cuda()) for o, i in cols]
+    off, ids = spread_sets(40, 3000, 28, seed=1)  # one batch: no narrower one to give way to
+    ref = oracle.all_pairs(off, ids)
+    plain = needed(lambda ctx: ctx.all_pairs(off, ids), ref)
+    a = Capped()
+    with jsim.Context(allocator=a) as ctx:
+        outs = ctx.all_pairs_batched(dev)
+        kept = a.now
+        assert kept > 64 << 20
+        a.total = max(a.peak, plain + kept - 4096)  # (the error word is part of both)
+        assert a.total < plain + kept - 256, "the two calls fit together: nothing is tested"
+        assert_same(ctx.all_pairs(off, ids), ref)
+        assert a.refused
+        again = ctx.all_pairs_batched(dev)
+        torch.cuda.synchronize()
+    for (C, s, J), (C2, s2, J2) in zip(outs, again):
+        assert torch.equal(C.view(torch.int32), C2.view(torch.int32)) and torch.equal(J, J2)
+    assert not a.live
