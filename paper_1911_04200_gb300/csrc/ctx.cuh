@@ -593,10 +593,15 @@ u64 dense_batch_rows(const jsim_ctx* ctx, u64 n, u64 N, u64 minid, u64 maxid, co
 // TC up to 128 samples is one 128 x 128 tile (the diagonal-tile kernel), above
 // it a padded one; it loads words by TMA, and rows that are not 16-byte
 // aligned take the byte-operand kernel, half as fast as POPC up to 96 samples.
+// POPC waits for nothing, so up to 96 samples, where it always could be had, it
+// is also taken under a bound on device waits that one accumulation of TC (at
+// most 2^22 bit-rows: 4 ms) comes near to.
+constexpr int kShortWaitMs = 100;
 int choose_variant(jsim_ctx* ctx, u64 n, u64 W, bool aligned = true)
 {
     (void)W;
-    if (!product_tc_supported(ctx->opt.device) || (n <= 96 && !aligned)) return JSIM_VARIANT_POPC;
+    const bool short_wait = ctx->opt.timeout_ms > 0 && ctx->opt.timeout_ms < kShortWaitMs;
+    if (!product_tc_supported(ctx->opt.device) || (n <= 96 && (!aligned || short_wait))) return JSIM_VARIANT_POPC;
     return n <= 128 ? JSIM_VARIANT_TC : JSIM_VARIANT_TC2;
 }
 
