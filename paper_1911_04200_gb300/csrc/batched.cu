@@ -41,9 +41,12 @@ struct Col {
 // stream would run them one after another.
 constexpr int kLanes = 4;
 // What a batch costs a lane whatever it holds, the lanes running beside one
-// another.  20 collections of 8 to 512 samples x 20,000 values in [0, 2^32),
-// the 13 below 256 sharing launches: 7.5 ms in 2^29-row batches, 6.8 in 2^30.
-constexpr double kWaveBatchMs = 0.06;
+// another: up to 1e7 values a collection take 2^30 rows, up to 4e6 2^31.
+// Values in [0, 2^32) unless said, whole calls in 2^29-row and wider batches:
+// 13 collections of 31 to 231 samples x 20,000 values 7.5 and 6.8 ms; 60 of 20
+// to 120 x 20,000 in [0, 2^30) 10.7 and 10.4; 12 of 150 to 255 x 60,000 (1.2e7
+// values or more each) 11.3 and 11.8, so these keep 2^29.
+constexpr double kWaveBatchMs = 0.04;
 
 // Everything one wave of collections needs on the device; kept alive by the
 // graph cache so a replay finds the same addresses.
