@@ -268,7 +268,10 @@ JSIM_API int jsim_partition_batches(uint64_t minid, uint64_t maxid, uint64_t bat
  * collection shape times the candidate products and remembers the fastest for
  * the context.  When every input and output is in device memory the launch
  * sequence is captured into a CUDA graph and later calls with the same
- * collections (same pointers and offsets) replay it after re-validating.
+ * collections (same pointers and offsets) replay it after re-validating; the
+ * context keeps the graph's buffers (the packed matrices and at most as much
+ * again, or 0.7 GB, of bitmaps) until a batched call on other collections, a
+ * refused allocation of another call, or jsim_destroy.
  * Errors: as jsim_all_pairs, plus JSIM_ERR_UNSUPPORTED when a collection's
  * value span needs more than 4096 row batches.
  */
@@ -524,7 +527,9 @@ JSIM_API int jsim_threshold(jsim_ctx* ctx, const double* J, uint64_t n, double t
  *   njobs       1..256; grid >= 1
  *   tile_n      the tile width: 256 (tiles of 128 x 256) or 128 (tiles of 128 x 128)
  *   stage_bits  bit-rows per stage: 256 (or 0), or 512 with tile_n 128 (the
- *               diagonal-only launch of the block-sparse path)
+ *               stages of the diagonal-tile product, which shares the units, segments
+ *               and accumulators but loads its words by TMA, not by the loads
+ *               replayed here)
  *   msg         receives a description of the first failed check (cap bytes, may be NULL)
  * Returns 0 when every check passes, JSIM_ERR_ARG for bad arguments, and a
  * positive check number otherwise.

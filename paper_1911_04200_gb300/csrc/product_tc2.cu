@@ -27,10 +27,10 @@
 // waits suspend in hardware instead of polling.  Measured (4096 samples,
 // 65,536 words; ms): FP8 operands in shared memory, 32-byte loads per row
 // 25.5; MXF4, same structure 15.5; whole-line loads 12.7; A in TMEM with
-// loads through registers 12.4, with cp.async 11.4; TMA 9.7 (7.7e15
+// loads through registers 12.4, with cp.async 11.4; TMA 9.6 (7.8e15
 // multiply-adds x 2 per second, of 10.3e15 for K = 64 MMAs at 2070 MHz; the
-// MMAs alone, with nothing unpacked, take 8.3 to 8.7).  n = 1024 and 65,536
-// words: 1.6 -> 0.72 ms.  Tried: six stages of 256 bit-rows 15.2 (the
+// MMAs alone, with nothing unpacked, take 8.3 to 8.7, so most of what is left
+// is the MMAs' own).  n = 1024 and 65,536 words: 1.6 -> 0.73 ms.  Tried: six stages of 256 bit-rows 15.2 (the
 // handshake between the CTAs is paid per stage); 16 unpacking warps 11.9 to
 // 12.4.
 //

@@ -1,8 +1,11 @@
 // Work schedule of the job-table tcgen05 product (product_tc.cu): which
 // (job, tile, stage) units a persistent CTA takes, which rows and words its
-// unpack threads read, and how its two TMEM accumulators are assigned.
+// unpack threads read, and how its two TMEM accumulators are assigned.  The
+// diagonal-tile product (product_tc_diag.cu) shares the units, their shares
+// and segments and the accumulators (stages of 512 bit-rows); its words come
+// by TMA instead of the per-thread reads.
 // Everything here is __host__ __device__, so the host-side schedule check
-// (jsim_check_tc_schedule) walks exactly the schedule the kernel runs.
+// (jsim_check_tc_schedule) walks exactly the schedule the kernels run.
 #pragma once
 #include "common.cuh"
 
@@ -14,7 +17,7 @@ constexpr int kM = 128;                        // A-side rows per tile
 // whose diagonal tiles unpack their rows once for both operands); the kernel
 // and these functions take it as a parameter `kn`.
 constexpr int kStageBits = 256;                // bit-rows per stage: two 128-byte swizzle atom columns
-                                               // (512 for diagonal-only launches: four; the functions
+                                               // (512 in the diagonal-tile product: the functions
                                                // below take the stage's words as a parameter)
 constexpr int kStageWords = kStageBits / 64;
 // a segment accumulates at most 2^22 bit-rows (exact FP32 counts)

@@ -85,7 +85,11 @@ double pair_product_ms(u64 n, double rows)
     return tt * (tt + 1.0) / 2.0 * 65536.0 * rows / kPairMacsPerMs;
 }
 // What the order of the samples takes, and with the sketch before it and the
-// classification that weighs it behind it (0.25 and 0.15).
+// classification that weighs it behind it (0.25 and 0.15).  With 0.4 against
+// 0.2 ms for the two, clade samples that stay dense are declined before the
+// sketch: 450 x 20,000 values over [0, 2^32) 1.49 -> 1.33 ms, 500 x 20,000 over
+// [0, 2^30) 1.23 -> 1.07; 900 x 20,000, 300 x 60,000 and 400 x 20,000 over
+// [0, 2^24), which go block-sparse, do so either way.
 double order_ms(u64 n) { return 0.05 + 0.7e-3 * (double)n; }
 double sketch_ms(u64 n) { return 0.4 + order_ms(n); }
 // Ranked ingest: at most this many values (a 32-bit row number is kept for
@@ -96,10 +100,15 @@ constexpr u64 kRankMaxValues = 1ull << 30;
 // range's work would go to samples with no value in it).
 constexpr int kWinLog = 16;
 constexpr double kWinMinValues = 0.5;
-// From this density the windowed ingest is taken whatever the other would
-// cost: over 2^32 rows the two cross at 4 to 5 values a window (1024 samples,
-// 2.1 a window: 11.4 ms windowed, 7.5 ranked; 6.2: 14.6 windowed, and the
-// ranked ingest alone would take 14).
+// From this density the windowed ingest is taken without weighing it against
+// the ranked one: its buffers do not grow with the number of values.  That is
+// not the faster choice everywhere: over 2^32 rows the two cross at 4 values a
+// window with one filter and at 5 or more with the two-or-more filter.  Whole
+// calls, windowed / ranked, in ms at 3, 4, 5 and 6 values a window:
+//   300 samples   4.2 / 3.7    4.4 / 4.3    4.5 / 4.8    4.8 / 5.3
+//   512           5.7 / 5.1    6.0 / 5.9    6.3 / 6.8    6.6 / 7.8
+//   1024         11.6 / 8.8   12.4 / 12.0  13.1 / 14.1  14.2 / 16.2
+//   1024, twice  13.8 / 9.9   14.7 / 11.7  15.3 / 13.8  16.2 / 15.9
 constexpr double kWinSureValues = 3.0;
 constexpr u64 kWinMaxBatch = 1ull << 30;
 
@@ -342,7 +351,8 @@ u64 feed_batch_rows(const jsim_ctx* ctx, u64 n, u64 N, u64 span)
 // The block-sparse path of jsim_all_pairs: JSIM_ERR_UNSUPPORTED where it does
 // not apply (more than kMaxTiles tiles, no tensor cores, a batch width that
 // is not a multiple of kMinClassRows); with may_decline, declined = true
-// when the sketch shows the product would not be halved (nothing written).
+// when the sketch shows that the order leaves more than 0.6 of the dense
+// product, or that the call is done sooner dense (nothing written).
 // With a feed, the values arrive piece by piece while the batches run (st
 // is validated when the last piece is in); with sv, the values are there and
 // their validation runs beside the sketch and the batches.  Either way
@@ -713,7 +723,7 @@ int all_pairs_sparse_with(jsim_ctx* ctx, Staged& st, void* C, uint64_t* sizes, d
         if (rc) return rc;
 
         if (may_decline && R_s) {
-            // the sketch range's rows by class: is the product at least halved?
+            // the sketch range's rows by class
             bool hn;
             u64 nx;
             rc = enqueue_classify(0, lo_s, std::max(ws, kMinClassRows));  // inside the first batch: same piece
