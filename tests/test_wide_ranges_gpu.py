@@ -63,3 +63,32 @@ def test_width_follows_the_values(gpu, name, make, wide, filter_min):
     np.testing.assert_array_equal(C.astype(np.uint64), Co)
     np.testing.assert_array_equal(J.view(np.uint64), Jo.view(np.uint64))
     assert rows > 1 << 28 if wide else rows <= 1 << 28
+
+
+@pytest.mark.parametrize("name,make,wide", CASES, ids=[c[0] for c in CASES])
+def test_block_sparse_over_the_same_ranges(gpu, name, make, wide):
+    off, ids = make()
+    Co, so, Jo = oracle.all_pairs(off, ids)
+    with jsim.Context(variant="sparse") as ctx:
+        C, s, J = ctx.all_pairs(off, ids)
+        st = ctx.stats()
+    assert st["variant"] == "sparse"
+    np.testing.assert_array_equal(s, so)
+    np.testing.assert_array_equal(C.astype(np.uint64), Co)
+    np.testing.assert_array_equal(J.view(np.uint64), Jo.view(np.uint64))
+    assert st["batch_rows"] > 1 << 28 if wide else st["batch_rows"] <= 1 << 28
+
+
+@pytest.mark.parametrize("values", [[0], [TOP - 1], [0, TOP - 1], [7] * 3, [1 << 40, (1 << 40) + 1],
+                                    [0, 1 << 32, 1 << 33, TOP - 1]])
+def test_fewer_values_than_probes(gpu, values):
+    segs = [sorted(values), [], sorted(set(values))[:1]]
+    off = np.array([0, len(segs[0]), len(segs[0]), len(segs[0]) + 1], dtype=np.uint64)
+    ids = np.array(segs[0] + segs[2], dtype=np.uint64)
+    Co, so, Jo = oracle.all_pairs(off, ids)
+    for variant in ("auto", "sparse"):
+        with jsim.Context(variant=variant) as ctx:
+            C, s, J = ctx.all_pairs(off, ids)
+        np.testing.assert_array_equal(s, so)
+        np.testing.assert_array_equal(C.astype(np.uint64), Co)
+        np.testing.assert_array_equal(J.view(np.uint64), Jo.view(np.uint64))
